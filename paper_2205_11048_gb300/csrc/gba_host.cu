@@ -169,6 +169,7 @@ struct gba_handle {
     int64_t accB;  // local batches of the step's messages so far
     int slot;      // its accumulator
     bool has_sum;  // some message of the step was kept
+    bool reverse;  // the next pass over the accumulator starts at its end
   };
   std::deque<EagerGroup> egroups;
   int n_acc = 0;
@@ -677,7 +678,7 @@ gba_status push_common(gba_handle* h, int64_t token, const gba_sparse_grad* per_
   if (eager) {  // the dense gradient joins its step's accumulator now
     if (new_group) {
       if (h->acc_ev_set[new_slot]) cudaStreamWaitEvent(h->stream, h->acc_ev[new_slot], 0);
-      h->egroups.push_back(gba_handle::EagerGroup{0, new_slot, false});
+      h->egroups.push_back(gba_handle::EagerGroup{0, new_slot, false, false});
     }
     gba_handle::EagerGroup& gr = h->egroups.back();
     const int64_t k_apply = h->k + (int64_t)h->egroups.size() - 1;
@@ -692,11 +693,12 @@ gba_status push_common(gba_handle* h, int64_t token, const gba_sparse_grad* per_
       float* hi = h->d_acc + (size_t)gr.slot * 2 * h->D_pad;
       {
         Timed tm(h, GBA_K_DENSE, h->stream);
-        launch_dense_accumulate(hi, hi + h->D_pad, src, h->D, f, !gr.has_sum, h->num_sms,
-                                h->stream);
+        launch_dense_accumulate(hi, hi + h->D_pad, src, h->D, f, !gr.has_sum, gr.reverse,
+                                h->num_sms, h->stream);
       }
       GBA_CUDA(h, cudaGetLastError());
       gr.has_sum = true;
+      gr.reverse = !gr.reverse;
     }
     gr.accB += local_batch;
     m.dense = nullptr;
@@ -1077,7 +1079,7 @@ int32_t gba_try_apply(gba_handle* h) {
       const float* hi = h->d_acc + (size_t)gr.slot * 2 * h->D_pad;
       {
         Timed tm(h, GBA_K_DENSE, h->side);
-        launch_dense_eager(da, hi, hi + h->D_pad, gr.has_sum, sink, h->num_sms, h->side);
+        launch_dense_eager(da, hi, hi + h->D_pad, gr.has_sum, gr.reverse, sink, h->num_sms, h->side);
       }
       cudaEventRecord(h->acc_ev[gr.slot], h->side);
       h->acc_ev_set[gr.slot] = true;

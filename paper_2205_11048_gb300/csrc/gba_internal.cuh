@@ -455,12 +455,13 @@ cudaError_t configure_dense();
 void launch_dense(const StepArgs& a, const DenseArgs& da, StepScratch sc, ErrSink err,
                   int64_t wait_ns, int num_sms, cudaStream_t s);
 
-// Eager dense aggregation: add f * g to a step's accumulator (first: start it),
-// and the step's update from the accumulator.
+// Eager dense aggregation: add f * g to a step's accumulator (first: start it;
+// reverse: from the last parameter down), and the step's update from the
+// accumulator.
 void launch_dense_accumulate(float* hi, float* lo, const float* g, int64_t D, float f, bool first,
-                             int num_sms, cudaStream_t s);
+                             bool reverse, int num_sms, cudaStream_t s);
 void launch_dense_eager(const DenseArgs& da, const float* hi, const float* lo, bool has_sum,
-                        ErrSink err, int num_sms, cudaStream_t s);
+                        bool reverse, ErrSink err, int num_sms, cudaStream_t s);
 
 void launch_init_table(float* w, float* s0, float* s1, int32_t* ver, int64_t rows, int32_t d,
                        int32_t kind, float init_acc, uint64_t seed, uint64_t tag,

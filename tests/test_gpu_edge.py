@@ -625,6 +625,28 @@ def test_eager_dense_equals_buffered(by_ref, rule):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("D", [1, 3, 5, 8_000_003, 9_000_000])
+def test_eager_dense_sizes(D):
+    """Push-time sums equal the buffered ones bit for bit at the edges of the
+    accumulate kernel: less than one float4, a ragged end, and sizes where the
+    direction alternates and only part of the accumulators is kept in cache."""
+    gen = torch.Generator(device="cuda").manual_seed(D)
+    grads = [torch.randn((D + 3) & ~3, generator=gen, device="cuda") for _ in range(4)]
+    outs = []
+    for eager in (False, True):
+        g = B.GBA([], D, B.opt_desc(1, 0.001), 4, 8, iota=3, seed=2)
+        if eager:
+            g.set_eager_dense(True)
+        for k in range(2):
+            for i, x in enumerate(grads):
+                g.push_ref(max(0, k - i), [], [], x[:D], 1)
+            assert g.try_apply() == 1
+        outs.append(g.dense())
+        g.close()
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
+
+
 def test_eager_dense_refusals_and_capacity():
     tables = [(100, 4, 0, 16, B.opt_desc())]
     g = B.GBA(tables, 1000, B.opt_desc(1, 0.001), 4, 64, seed=1, iota=3, drop_latest=1)
