@@ -579,6 +579,50 @@ float message_weight(const gba_handle* h, int64_t k_apply, int64_t token) {
   return s < (int64_t)h->h_wtab.size() ? h->h_wtab[s] : 0.f;
 }
 
+// Whether a kernel on the handle's device may read p itself: memory of that
+// device, or managed.  (Host memory goes through the copy engine, which reads
+// it at the link's rate.)
+bool device_readable(const gba_handle* h, const void* p) {
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (at.type == cudaMemoryTypeDevice && at.device == h->device) ||
+         at.type == cudaMemoryTypeManaged;
+}
+
+// The copies of one push: arrays that the device can read are gathered and
+// copied by one launch (flush), the others are enqueued one by one.
+struct PushCopies {
+  gba_handle* h;
+  CopyList cl;
+  explicit PushCopies(gba_handle* h_) : h(h_) { cl.n = 0; }
+  cudaError_t add(void* dst, const void* src, size_t bytes) {
+    if (bytes == 0) return cudaSuccess;
+    if (!device_readable(h, src)) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, h->stream);
+    if (cl.n == COPY_MAX) {
+      const cudaError_t e = flush();
+      if (e != cudaSuccess) return e;
+    }
+    cl.src[cl.n] = src;
+    cl.dst[cl.n] = dst;
+    cl.bytes[cl.n++] = bytes;
+    return cudaSuccess;
+  }
+  cudaError_t flush() {
+    if (cl.n == 0) return cudaSuccess;
+    // a launch needs the stream's device current; a copy did not
+    int dev = h->device;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && dev != h->device) e = cudaSetDevice(h->device);
+    if (e == cudaSuccess) e = launch_push_copy(cl, h->stream);
+    if (dev != h->device) cudaSetDevice(dev);
+    cl.n = 0;
+    return e;
+  }
+};
+
 gba_status push_common(gba_handle* h, int64_t token, const gba_sparse_grad* per_table,
                        const float* dense_grad, int32_t local_batch, bool copy) {
   if (!h) return GBA_E_ARG;
@@ -642,6 +686,7 @@ gba_status push_common(gba_handle* h, int64_t token, const gba_sparse_grad* per_
       }
       m.arena_v[t] = v;
     }
+    PushCopies copies(h);
     for (int t = 0; t < h->T; ++t) {
       const int64_t n = per_table[t].n;
       Arena& ar = h->tables[t].arena;
@@ -650,23 +695,19 @@ gba_status push_common(gba_handle* h, int64_t token, const gba_sparse_grad* per_
       m.ids[t] = ar.ids + p;
       m.rows[t] = ar.rows + p * dim;
       m.n[t] = n;
-      if (n > 0) {
-        GBA_CUDA(h, cudaMemcpyAsync(ar.ids + p, per_table[t].ids, n * sizeof(int64_t),
-                                    cudaMemcpyDefault, h->stream));
-        GBA_CUDA(h, cudaMemcpyAsync(ar.rows + p * dim, per_table[t].rows,
-                                    n * dim * sizeof(float), cudaMemcpyDefault, h->stream));
-      }
+      GBA_CUDA(h, copies.add(ar.ids + p, per_table[t].ids, n * sizeof(int64_t)));
+      GBA_CUDA(h, copies.add(ar.rows + p * dim, per_table[t].rows, n * dim * sizeof(float)));
     }
     if (h->D > 0 && !eager) {
       const int32_t slot = (h->slot_head + h->slot_count) % h->max_buf;
       float* dst = h->dense_ring + (size_t)slot * h->D_pad;
-      GBA_CUDA(h, cudaMemcpyAsync(dst, dense_grad, h->D * sizeof(float), cudaMemcpyDefault,
-                                  h->stream));
+      GBA_CUDA(h, copies.add(dst, dense_grad, h->D * sizeof(float)));
       h->slot_count++;
       m.dense = dst;
     } else {
       m.dense = nullptr;
     }
+    GBA_CUDA(h, copies.flush());
   } else {
     for (int t = 0; t < h->T; ++t) {
       m.ids[t] = per_table[t].ids;
@@ -685,7 +726,8 @@ gba_status push_common(gba_handle* h, int64_t token, const gba_sparse_grad* per_
     const float f = message_weight(h, k_apply, token);
     if (f > 0.f) {
       const float* src = dense_grad;
-      if (copy) {
+      // summed where it lies, if the kernel can read it there (aligned float4)
+      if (copy && !(((uintptr_t)dense_grad & 15u) == 0 && device_readable(h, dense_grad))) {
         GBA_CUDA(h, cudaMemcpyAsync(h->d_stage_dense, dense_grad, h->D * sizeof(float),
                                     cudaMemcpyDefault, h->stream));
         src = h->d_stage_dense;

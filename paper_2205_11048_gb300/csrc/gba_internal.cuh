@@ -455,6 +455,18 @@ cudaError_t configure_dense();
 void launch_dense(const StepArgs& a, const DenseArgs& da, StepScratch sc, ErrSink err,
                   int64_t wait_ns, int num_sms, cudaStream_t s);
 
+// Arrays copied by one launch: a pushed message's ids, gradient rows and dense
+// gradient (at most COPY_MAX of them, each smaller than 2^44 bytes).
+constexpr int COPY_MAX = 32;
+struct CopyList {
+  const void* src[COPY_MAX];
+  void* dst[COPY_MAX];
+  uint64_t bytes[COPY_MAX];
+  uint32_t first[COPY_MAX];  // first block of each array (set by launch_push_copy)
+  int32_t n;
+};
+cudaError_t launch_push_copy(CopyList cl, cudaStream_t s);
+
 // Eager dense aggregation: add f * g to a step's accumulator (first: start it;
 // reverse: from the last parameter down), and the step's update from the
 // accumulator.

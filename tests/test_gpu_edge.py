@@ -625,6 +625,57 @@ def test_eager_dense_equals_buffered(by_ref, rule):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("where", ["device", "pinned", "pageable"])
+@pytest.mark.parametrize("shift", [0, 1, 2])
+@pytest.mark.parametrize("eager", [False, True])
+def test_copying_push_of_any_alignment(where, shift, eager):
+    """A copying push takes arrays at any element offset, on the device or in
+    host memory, empty ones and more arrays than one copy launch holds among
+    them: the state is that of the same messages pushed by reference."""
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    dims = [1, 4, 7, 64] + [3] * 14  # 2 * 18 + 1 arrays
+    ns = [5, 4099, 0, 70] + [9] * 14
+    D = 5003
+    tables = [(50, d, 0, 4099, B.opt_desc(0, 0.01)) for d in dims]
+    msgs = []
+    for m in range(2):
+        ids = [torch.randint(0, 50, (n,), generator=gen, device="cuda") for n in ns]
+        rows = [torch.randn(n, d, generator=gen, device="cuda") for n, d in zip(ns, dims)]
+        msgs.append((ids, rows, torch.randn((D + 3) & ~3, generator=gen, device="cuda")[:D]))
+
+    def moved(x):  # the same values `shift` elements past an allocation's start
+        buf = torch.empty(x.numel() + shift, dtype=x.dtype,
+                          device="cuda" if where == "device" else "cpu")
+        if where == "pinned":
+            buf = buf.pin_memory()
+        out = buf[shift:].view(x.shape)
+        out.copy_(x)
+        return out
+
+    states = []
+    for copying in (False, True):
+        g = B.GBA(tables, D, B.opt_desc(1, 0.001), 2, 4, iota=3, seed=4)
+        if eager:
+            g.set_eager_dense(True)
+        keep = []
+        for ids, rows, dense in msgs:
+            if copying:
+                a = ([moved(x) for x in ids], [moved(x) for x in rows], moved(dense))
+                keep.append(a)
+                torch.cuda.synchronize()
+                g.push(0, *a, 1)
+            else:
+                torch.cuda.synchronize()
+                g.push_ref(0, ids, rows, dense, 1)
+        assert g.try_apply() == 1
+        g.sync()
+        states.append([t for t in g.dense() if t is not None] +
+                      [t for i in range(len(dims)) for t in g.table(i) if t is not None])
+        g.close()
+    for a, b in zip(*states):
+        assert torch.equal(a, b)
+
+
 @pytest.mark.parametrize("D", [1, 3, 5, 8_000_003, 9_000_000])
 def test_eager_dense_sizes(D):
     """Push-time sums equal the buffered ones bit for bit at the edges of the
