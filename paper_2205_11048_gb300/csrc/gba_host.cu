@@ -144,8 +144,8 @@ struct gba_handle {
   char* d_step_scratch[SLOTS] = {};
   StepScratch sc[SLOTS] = {};
   // row-kernel buffers (apply stream only), grown with n_cap
-  uint4* d_rr = nullptr;                   // row records, per table nbase[t] + t
-  const float** d_kl = nullptr;            // kept list, per table nbase[t]
+  uint4* d_rr = nullptr;                   // row records
+  const float** d_kl = nullptr;            // kept list
   float* d_kw = nullptr;                   // kept weights
   unsigned long long* d_scan_status = nullptr;
   uint4* d_long_rows = nullptr;
@@ -154,8 +154,7 @@ struct gba_handle {
   uint2* d_items = nullptr;
   float* d_part_hi = nullptr;
   float* d_part_lo = nullptr;
-  uint32_t* d_seg_total = nullptr;         // [T] rows of each table in the last step
-  int d_max = 1;
+  uint32_t* d_ustart = nullptr;            // [T + 1] first row record of each table in the last step
 
   float* d_wtab = nullptr;    // decay weights lambda^s (decay 1)
   int32_t n_wtab = 0;
@@ -329,7 +328,7 @@ void free_all(gba_handle* h) {
   }
   for (void* p : {(void*)h->d_rr, (void*)h->d_kl, (void*)h->d_kw, (void*)h->d_scan_status,
                   (void*)h->d_long_rows, (void*)h->d_long_done, (void*)h->d_items,
-                  (void*)h->d_part_hi, (void*)h->d_part_lo, (void*)h->d_seg_total,
+                  (void*)h->d_part_hi, (void*)h->d_part_lo, (void*)h->d_ustart,
                   (void*)h->d_small_rows})
     cudaFree(p);
   cudaFree(h->d_err);
@@ -518,8 +517,8 @@ gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
     }
     h->n_cap = cap;
     h->status_tiles = tiles;
-    // row-kernel buffers: a record per possible row (and one per table for the
-    // totals), a kept-list entry per occurrence, look-back words per scan tile,
+    // row-kernel buffers: a record per possible row (and one for the totals),
+    // a kept-list entry per occurrence, look-back words per scan tile,
     // long rows and their chunks
     for (void* p : {(void*)h->d_rr, (void*)h->d_kl, (void*)h->d_kw, (void*)h->d_scan_status,
                     (void*)h->d_long_rows, (void*)h->d_long_done, (void*)h->d_items,
@@ -535,8 +534,10 @@ gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
     h->d_items = nullptr;
     const int64_t stiles = scan_tiles(cap);
     const int64_t long_cap = cap / (LONG_ROW + 1) + h->T + 1;
-    const int64_t items_cap = cap / LONG_CHUNK + long_cap;
-    const int64_t parts_cap = 2 * (cap / LONG_CHUNK) + h->T + 1;
+    const int64_t items_cap = cap / MIN_CHUNK + long_cap;
+    int64_t part_floats = 1;  // of the widest range of tables
+    for (const TableState& ts : h->tables)
+      part_floats = std::max(part_floats, long_parts(cap, ts.desc.dim) * ts.desc.dim);
     GBA_CUDA(h, cudaMalloc(&h->d_rr, (size_t)(cap + h->T + 1) * sizeof(uint4)));
     GBA_CUDA(h, cudaMalloc(&h->d_kl, (size_t)cap * sizeof(float*)));
     GBA_CUDA(h, cudaMalloc(&h->d_kw, (size_t)cap * sizeof(float)));
@@ -546,8 +547,8 @@ gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
     GBA_CUDA(h, cudaMalloc(&h->d_small_rows, (size_t)long_cap * sizeof(uint4)));
     GBA_CUDA(h, cudaMalloc(&h->d_long_done, (size_t)long_cap * sizeof(uint32_t)));
     GBA_CUDA(h, cudaMalloc(&h->d_items, (size_t)items_cap * sizeof(uint2)));
-    GBA_CUDA(h, cudaMalloc(&h->d_part_hi, (size_t)parts_cap * h->d_max * sizeof(float)));
-    GBA_CUDA(h, cudaMalloc(&h->d_part_lo, (size_t)parts_cap * h->d_max * sizeof(float)));
+    GBA_CUDA(h, cudaMalloc(&h->d_part_hi, (size_t)part_floats * sizeof(float)));
+    GBA_CUDA(h, cudaMalloc(&h->d_part_lo, (size_t)part_floats * sizeof(float)));
   }
   return GBA_OK;
 }
@@ -854,7 +855,6 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
       while (slots < ts.desc.rows) slots *= 2;
       ts.desc.rows = slots;
     }
-    h->d_max = std::max(h->d_max, (int)tables[t].dim);
   }
 
   auto dev_alloc = [&](void** p, size_t bytes) -> bool {
@@ -891,7 +891,8 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
   {
     const size_t M = (size_t)max_buffered_msgs, T = (size_t)n_tables;
     h->meta_bytes = align16(M * 8) + align16(M * 8) + align16(T * (M + 1) * 4) +
-                    align16(T * M * 8) + align16(T * M * 8) + align16((T + 1) * 8);
+                    align16(T * M * 8) + align16(T * M * 8) + align16((T + 1) * 8) +
+                    align16(T * sizeof(SegTable));
     for (int b = 0; b < SLOTS; ++b)
       if (!dev_alloc((void**)&h->d_meta[b], h->meta_bytes)) return fail(GBA_E_OOM);
     for (int i = 0; i < META_SLOTS; ++i) {
@@ -928,7 +929,7 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
       sc.fw = (float*)p;
     }
   }
-  if (!dev_alloc((void**)&h->d_seg_total, (size_t)std::max(h->T, 1) * 4)) return fail(GBA_E_OOM);
+  if (!dev_alloc((void**)&h->d_ustart, (size_t)(h->T + 1) * 4)) return fail(GBA_E_OOM);
   if (rule.decay == 1) {  // lambda^s as s products in double, rounded once, s = 0 .. iota
     h->n_wtab = rule.iota + 1;
     std::vector<float>& wt = h->h_wtab;
@@ -1051,7 +1052,8 @@ int32_t gba_try_apply(gba_handle* h) {
   };
   const size_t o_tok = section(Mx * 8), o_dense = section(Mx * 8),
                o_off = section((size_t)T * (Mx + 1) * 4), o_ids = section((size_t)T * Mx * 8),
-               o_rows = section((size_t)T * Mx * 8), o_nbase = section((size_t)(T + 1) * 8);
+               o_rows = section((size_t)T * Mx * 8), o_nbase = section((size_t)(T + 1) * 8),
+               o_tabs = section((size_t)T * sizeof(SegTable));
   int64_t* tok = (int64_t*)(hp + o_tok);
   const float** dptr = (const float**)(hp + o_dense);
   uint32_t* moff = (uint32_t*)(hp + o_off);
@@ -1075,6 +1077,26 @@ int32_t gba_try_apply(gba_handle* h) {
     moff[(size_t)t * (M + 1) + M] = run;
   }
   for (int t = 0; t <= T; ++t) nb[t] = nbase[t];
+  SegTable* tabs = (SegTable*)(hp + o_tabs);
+  for (int t = 0; t < T; ++t) {
+    const TableState& ts = h->tables[t];
+    const int64_t Nt = nbase[t + 1] - nbase[t];
+    SegTable tb{};
+    tb.w = ts.w;
+    tb.s0 = ts.s0;
+    tb.s1 = ts.s1;
+    tb.ver = ts.ver;
+    tb.d = ts.desc.dim;
+    tb.t = t;
+    tb.key_base = ts.key_base;
+    tb.rows = (uint32_t)ts.desc.rows;
+    tb.nb = (uint32_t)nbase[t];
+    tb.n = (uint32_t)Nt;
+    tb.mscale = (float)M / (float)std::max<int64_t>(1, Nt);
+    tb.opt = make_opt_step(ts.desc.opt, ts.bpow1 * (double)ts.desc.opt.beta1,
+                           ts.bpow2 * (double)ts.desc.opt.beta2);
+    tabs[t] = tb;
+  }
   GBA_CUDA(h, cudaMemcpyAsync(dmeta, hp, h->meta_bytes, cudaMemcpyHostToDevice, h->sorts));
   cudaEventRecord(h->meta_ev[slot], h->sorts);
 
@@ -1156,62 +1178,48 @@ int32_t gba_try_apply(gba_handle* h) {
     }
     cudaEventRecord(h->ev_sorted[b], h->sorts);
     cudaStreamWaitEvent(h->applys, h->ev_sorted[b], 0);
-    for (int t = 0; t < T; ++t) {
-      const int64_t Nt = nbase[t + 1] - nbase[t];
-      if (Nt == 0) continue;
-      TableState& ts = h->tables[t];
-      const double p1 = ts.bpow1 * (double)ts.desc.opt.beta1;
-      const double p2 = ts.bpow2 * (double)ts.desc.opt.beta2;
-      SegTable tb{};
-      tb.w = ts.w;
-      tb.s0 = ts.s0;
-      tb.s1 = ts.s1;
-      tb.ver = ts.ver;
-      tb.d = ts.desc.dim;
-      tb.t = t;
-      tb.key_base = ts.key_base;
-      tb.rows = ts.desc.rows;
-      tb.pos_begin = nbase[t];
-      tb.pos_end = nbase[t + 1];
-      tb.opt = make_opt_step(ts.desc.opt, p1, p2);
-      if (++h->epoch == 0u) h->epoch = 1u;
-      SegOut so{};
-      so.rr = h->d_rr + nbase[t] + t;
-      so.kl = h->d_kl + nbase[t];
-      so.kw = h->d_kw + nbase[t];
-      so.status = h->d_scan_status;
-      so.epoch = h->epoch;
-      so.ticket = sc.seg_ticket + 8 * t;
-      so.n_long = sc.seg_ticket + 8 * t + 1;
-      so.n_items = sc.seg_ticket + 8 * t + 2;
-      so.n_parts = sc.seg_ticket + 8 * t + 3;
-      so.item_ticket = sc.seg_ticket + 8 * t + 4;
-      so.total = h->d_seg_total + t;
-      so.long_rows = h->d_long_rows;
-      so.long_done = h->d_long_done;
-      so.items = h->d_items;
-      so.part_hi = h->d_part_hi;
-      so.part_lo = h->d_part_lo;
-      so.pstride = h->d_max;
-      so.small_rows = h->d_small_rows;
-      so.n_small = sc.seg_ticket + 8 * t + 5;
-      so.small_ticket = sc.seg_ticket + 8 * t + 6;
-      {
-        Timed tm(h, GBA_K_SEG_SCAN, h->applys);
-        launch_seg_scan(a, tb, so, h->d_keys[b][final_buf], h->d_vals[b][final_buf], h->d_stats,
-                        sink, h->wait_ns, h->applys);
-      }
-      {
-        Timed tm(h, GBA_K_SEG_SCAN, h->applys);
-        launch_row_classify(a, tb, so, sink, h->num_sms, h->applys);
-      }
+    if (++h->epoch == 0u) h->epoch = 1u;
+    SegOut so{};
+    so.rr = h->d_rr;
+    so.kl = h->d_kl;
+    so.kw = h->d_kw;
+    so.status = h->d_scan_status;
+    so.epoch = h->epoch;
+    so.ticket = sc.seg_ticket;
+    so.ustart = h->d_ustart;
+    so.long_rows = h->d_long_rows;
+    so.long_done = h->d_long_done;
+    so.items = h->d_items;
+    so.part_hi = h->d_part_hi;
+    so.part_lo = h->d_part_lo;
+    so.small_rows = h->d_small_rows;
+    const SegTable* d_tabs = (const SegTable*)(dmeta + o_tabs);
+    {
+      Timed tm(h, GBA_K_SEG_SCAN, h->applys);
+      launch_seg_scan(a, tabs[0], d_tabs, so, h->d_keys[b][final_buf], h->d_vals[b][final_buf],
+                      h->d_stats, sink, h->wait_ns, h->applys);
+    }
+    // one pair of row kernels per range of consecutive tables of one width and
+    // optimizer
+    for (int t0 = 0, t1; t0 < T; t0 = t1) {
+      for (t1 = t0 + 1; t1 < T && tabs[t1].d == tabs[t0].d && tabs[t1].opt.kind == tabs[t0].opt.kind;)
+        ++t1;
+      const RowRange r{t0, t1, nbase[t1] - nbase[t0], tabs[t0]};
+      if (r.n == 0) continue;
+      uint32_t* counters = sc.seg_ticket + 8 * t0;
+      so.n_long = counters + 1;
+      so.n_items = counters + 2;
+      so.n_parts = counters + 3;
+      so.item_ticket = counters + 4;
+      so.n_small = counters + 5;
+      so.small_ticket = counters + 6;
       {
         Timed tm(h, GBA_K_ROW_APPLY, h->applys);
-        launch_row_apply(a, tb, so, h->d_stats, sink, h->num_sms, h->applys);
+        launch_row_apply(a, r, d_tabs, so, h->d_stats, sink, h->num_sms, h->applys);
       }
       {
         Timed tm(h, GBA_K_ROW_LONG, h->applys);
-        launch_row_long(a, tb, so, h->d_stats, sink, h->num_sms, h->applys);
+        launch_row_long(a, r, d_tabs, so, h->d_stats, sink, h->num_sms, h->applys);
       }
     }
   }
@@ -1422,24 +1430,24 @@ gba_status gba_debug_segments(gba_handle* h, int64_t cap, int32_t* table, int64_
   GBA_CUDA(h, sync_all(h));
   // the step's row records, table by table: (row, prefixes of kept occurrences
   // and of (message, row) pairs at the row's head), closed by the totals
-  std::vector<uint32_t> U(h->T, 0u);
-  if (h->T > 0 && h->last_N > 0)
-    GBA_CUDA(h, cudaMemcpy(U.data(), h->d_seg_total, h->T * sizeof(uint32_t),
+  std::vector<uint32_t> us((size_t)h->T + 1, 0u);
+  std::vector<uint4> rr;
+  if (h->T > 0 && h->last_N > 0) {
+    GBA_CUDA(h, cudaMemcpy(us.data(), h->d_ustart, us.size() * sizeof(uint32_t),
                            cudaMemcpyDeviceToHost));
+    rr.resize((size_t)us[h->T] + 1);
+    GBA_CUDA(h, cudaMemcpy(rr.data(), h->d_rr, rr.size() * sizeof(uint4), cudaMemcpyDeviceToHost));
+  }
   int64_t u_all = 0;
   for (int t = 0; t < h->T; ++t) {
-    const int64_t Nt = h->last_nbase[t + 1] - h->last_nbase[t];
-    if (Nt == 0) continue;
-    std::vector<uint4> rr((size_t)U[t] + 1);
-    GBA_CUDA(h, cudaMemcpy(rr.data(), h->d_rr + h->last_nbase[t] + t, rr.size() * sizeof(uint4),
-                           cudaMemcpyDeviceToHost));
+    if (us[t + 1] == us[t]) continue;
     std::vector<unsigned long long> keys;  // HASH tables report the id of each slot
     if (h->tables[t].desc.id_mode == GBA_ID_HASH) {
       keys.resize((size_t)h->tables[t].desc.rows);
       GBA_CUDA(h, cudaMemcpy(keys.data(), h->tables[t].keys, keys.size() * 8,
                              cudaMemcpyDeviceToHost));
     }
-    for (uint32_t u = 0; u < U[t]; ++u, ++u_all) {
+    for (uint32_t u = us[t]; u < us[t + 1]; ++u, ++u_all) {
       if (u_all >= cap) continue;
       if (table) table[u_all] = t;
       if (row) row[u_all] = keys.empty() ? (int64_t)rr[u].x : (int64_t)keys[rr[u].x];

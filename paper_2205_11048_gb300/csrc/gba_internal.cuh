@@ -198,9 +198,10 @@ struct OptStep {
 };
 
 // Adagrad and Adam, one IEEE float operation at a time in a fixed order.
-__device__ __forceinline__ void opt_update(const OptStep& o, float& w, float& s0, float& s1,
-                                           float g) {
-  if (o.kind == 0) {
+template <bool ADAM>
+__device__ __forceinline__ void opt_update_as(const OptStep& o, float& w, float& s0, float& s1,
+                                              float g) {
+  if (!ADAM) {
     float gg = __fmul_rn(g, g);
     float an = __fadd_rn(s0, gg);
     float step = __fmul_rn(o.lr, g);
@@ -219,6 +220,13 @@ __device__ __forceinline__ void opt_update(const OptStep& o, float& w, float& s0
     s1 = vn;
     w = __fsub_rn(w, __fdiv_rn(num, den));
   }
+}
+__device__ __forceinline__ void opt_update(const OptStep& o, float& w, float& s0, float& s1,
+                                           float g) {
+  if (o.kind == 0)
+    opt_update_as<false>(o, w, s0, s1, g);
+  else
+    opt_update_as<true>(o, w, s0, s1, g);
 }
 
 // Error-free transformation of a + b (Knuth's TwoSum): s + e == a + b exactly.
@@ -280,8 +288,9 @@ struct StepScratch {
   int32_t* kept_list;      // [M] indices of kept messages, in pop order
   int32_t* n_kept;         // [1]
   uint32_t* step_err;      // [1] failures of this step
-  uint32_t* seg_ticket;    // [T][8] per table: scan tile tickets, long rows, their items,
-                           // chunk-sum slots, item tickets, unused
+  uint32_t* seg_ticket;    // [T][8]: word 0 scan tile tickets; words 8 t0 + 1 .. 6, for the
+                           // range of tables from t0: long rows, their items, chunk-sum
+                           // slots, item tickets, small rows, small-row tickets
   float* fw;               // [M] message weights of the dense sum (decay 1; 1 or 0 otherwise)
 };
 
@@ -359,6 +368,7 @@ void launch_onesweep(const StepArgs& a, bool first, int pass, const uint32_t* ke
 
 int sort_tiles(int64_t N);
 
+// One table as the row kernels see it.
 struct SegTable {
   float* w;
   float* s0;
@@ -367,77 +377,88 @@ struct SegTable {
   int32_t d;
   int32_t t;
   uint32_t key_base;
-  int32_t pad;
-  int64_t rows;                // V of the table
-  int64_t pos_begin, pos_end;  // range of the sorted array holding this table's keys
+  uint32_t rows;  // V of the table
+  uint32_t nb;    // first position of its keys in the sorted array, and first occurrence
+  uint32_t n;     // how many it has
+  float mscale;   // messages over occurrences
+  uint32_t pad;
   OptStep opt;
+  uint32_t pad2;
+};
+static_assert(sizeof(SegTable) % 8 == 0, "copied as words, followed by 8-byte values");
+
+// Consecutive tables of one width and optimizer, handled by one launch of each
+// row kernel.
+struct RowRange {
+  int32_t t0, t1;  // tables [t0, t1)
+  int64_t n;       // their occurrences
+  SegTable first;  // table t0
 };
 
 // Buffers of the row kernels (one set, used in stream order by the apply
-// stream; every table of a step uses its own ranges of rr / kl / kw).
-//  rr[u]   row u of the table in sorted order: (row x, and the exclusive
-//          prefixes at its head of kept occurrences K, (message, row) pairs C
-//          and kept pairs CK); rr[U] holds the totals, so row u's kept
+// stream).
+//  rr[u]   row u in sorted order over all tables: (row x of its table, and the
+//          exclusive prefixes at its head of kept occurrences K, (message, row)
+//          pairs C and kept pairs CK); rr[U] holds the totals, so row u's kept
 //          occurrences are kl[rr[u].K .. rr[u+1].K), c_x = rr[u+1].C - rr[u].C
 //  kl[j]   address of the j-th kept occurrence's gradient row, sorted by row
-//  kw[j]   its weight f (1 under Eq. (1))
+//  kw[j]   its weight f (not written under Eq. (1), where it is 1)
+//  ustart[t]  first row record of table t; ustart[T] = U
+// The lists and their counters belong to the range of tables being applied.
 struct SegOut {
-  uint4* rr;                   // this table's range
-  const float** kl;            // this table's range
-  float* kw;                   // this table's range
+  uint4* rr;
+  const float** kl;
+  float* kw;
   unsigned long long* status;  // [tiles][4] look-back words of the scan
   uint32_t epoch;              // tag of this launch's look-back words
   uint32_t* ticket;            // scan tile tickets (cleared by K1)
-  uint32_t* n_long;            // rows with more than LONG_ROW kept occurrences (cleared by K1)
+  uint32_t* ustart;            // [T + 1]
+  uint32_t* n_long;            // rows with more than SMALL_MAX kept occurrences (cleared by K1)
   uint32_t* n_items;           // chunks of those rows (cleared by K1)
   uint32_t* n_parts;           // chunk-sum slots of rows split into chunks (cleared by K1)
   uint32_t* item_ticket;       // items claimed by warps of the long-row kernel (cleared by K1)
-  uint32_t* total;             // this table's U (written by the last scan tile)
   uint4* long_rows;            // [n_long] (u, first kept, kept count, first chunk-sum slot)
   uint32_t* long_done;         // [n_long] chunks of the row finished
   uint2* items;                // [n_items] (long row, chunk)
-  float* part_hi;              // [n_parts][pstride] compensated chunk sums
+  float* part_hi;              // [n_parts][d] compensated chunk sums
   float* part_lo;
-  int32_t pstride;
-  uint4* small_rows;           // [n_small] (row, first kept, kept count, denominator bits)
-  uint32_t* n_small;           // long rows of at most SMALL_MAX kept occurrences (cleared by K1)
+  uint4* small_rows;           // [n_small] (row, first kept, table << 8 | kept count, denominator)
+  uint32_t* n_small;           // rows of LONG_ROW + 1 .. SMALL_MAX kept occurrences (cleared by K1)
   uint32_t* small_ticket;      // small rows claimed by the long-row kernel (cleared by K1)
 };
 
-// Rows with at most LONG_ROW kept occurrences are applied by one lane group
-// each with all their gradient rows staged in shared memory; longer rows by a
-// whole warp each, in chunks of LONG_CHUNK kept occurrences.
+// Rows with at most LONG_ROW kept occurrences are applied by k_row_apply,
+// rows of at most SMALL_MAX by one lane group of k_row_long each, longer ones
+// in chunks.
 constexpr int LONG_ROW = 4;
-#ifndef GBA_LONG_CHUNK
-#define GBA_LONG_CHUNK 128
-#endif
-constexpr int LONG_CHUNK = GBA_LONG_CHUNK;
-// Long rows of at most SMALL_MAX kept occurrences are applied by one lane
-// group each, with all their gradient rows staged in shared memory.
 #ifndef GBA_SMALL_MAX
 #define GBA_SMALL_MAX 32
 #endif
 constexpr int SMALL_MAX = GBA_SMALL_MAX;
+static_assert(SMALL_MAX < 256, "a small row's count shares a word with its table");
+constexpr int MIN_CHUNK = 128;  // least kept occurrences per chunk of a long row
 #ifndef GBA_SCAN_TILE
 #define GBA_SCAN_TILE 2048
 #endif
 constexpr int SCAN_TILE = GBA_SCAN_TILE;  // sorted positions per segment-scan tile
 
 int64_t scan_tiles(int64_t N);
+// The most chunk-sum slots that n occurrences of rows of width d can need.
+int64_t long_parts(int64_t n, int d);
 
-void launch_seg_scan(const StepArgs& a, const SegTable& tb, const SegOut& so, const uint32_t* keys,
-                     const uint32_t* vals, DevStats* stats, ErrSink err, int64_t wait_ns,
+// tb0: the first table; tabs: all of them, on the device.
+void launch_seg_scan(const StepArgs& a, const SegTable& tb0, const SegTable* tabs,
+                     const SegOut& so, const uint32_t* keys, const uint32_t* vals,
+                     DevStats* stats, ErrSink err, int64_t wait_ns, cudaStream_t s);
+
+// The range's rows with few kept occurrences; lists the others for
+// launch_row_long, which comes next on the stream.
+void launch_row_apply(const StepArgs& a, const RowRange& r, const SegTable* tabs,
+                      const SegOut& so, DevStats* stats, ErrSink err, int num_sms,
+                      cudaStream_t s);
+void launch_row_long(const StepArgs& a, const RowRange& r, const SegTable* tabs,
+                     const SegOut& so, DevStats* stats, ErrSink err, int num_sms,
                      cudaStream_t s);
-
-void launch_row_apply(const StepArgs& a, const SegTable& tb, const SegOut& so, DevStats* stats,
-                      ErrSink err, int num_sms, cudaStream_t s);
-
-void launch_row_long(const StepArgs& a, const SegTable& tb, const SegOut& so, DevStats* stats,
-                     ErrSink err, int num_sms, cudaStream_t s);
-
-// Lists the long rows and their chunks (after the scan, before both row kernels).
-void launch_row_classify(const StepArgs& a, const SegTable& tb, const SegOut& so, ErrSink err,
-                         int num_sms, cudaStream_t s);
 
 struct DenseArgs {
   float* w;

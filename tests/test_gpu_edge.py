@@ -326,6 +326,67 @@ def test_kept_count_boundaries_of_the_row_kernels(dim, rule):
     run_custom(cfg, steps, rule=rule)
 
 
+@pytest.mark.parametrize("dim,chunk", [(4, 2048), (8, 1024), (13, 128), (16, 512), (28, 256), (132, 128)])
+def test_chunk_boundaries_of_long_rows(dim, chunk):
+    """Rows with kept occurrences on each side of one and of several chunks,
+    whose size depends on the width, and one with more chunks than a lane group
+    merges at a time."""
+    counts = [chunk - 1, chunk, chunk + 1, 2 * chunk, 2 * chunk + 1, 37 * chunk + 3, 1, 33]
+    M, D = 3, 5
+    rng = np.random.default_rng(dim)
+    cfg = cfg_of([(len(counts) + 2, dim, 0, 0)], D=D, G=M, iota=1)
+
+    def batch(k):
+        ids = rng.permutation(np.repeat(np.arange(len(counts)), counts))
+        cut = sorted(rng.integers(0, len(ids), M - 1))
+        return [msg(max(0, k - 2 * (m == 1)), [part], [dim], D, scale=0.001)
+                for m, part in enumerate(np.split(ids, cut))]
+
+    run_custom(cfg, [batch(0), batch(1), batch(2)], max_ids=60 * chunk + 200)
+
+
+def test_tables_that_share_launches():
+    """Runs of tables of one width and optimizer, other widths and optimizers
+    between them, and tables without ids first, last, between and alone in
+    their run: rows of every length in each, against the oracle."""
+    shape = [(40, 8, 0, 0), (30, 8, 0, 0), (5000, 8, 1, 0), (20, 8, 0, 1), (25, 8, 0, 1), (60, 5, 0, 0),
+             (9, 64, 0, 0), (33, 8, 0, 0), (50, 8, 0, 0)]
+    dims = [s[1] for s in shape]
+    cfg = cfg_of(shape, D=7, G=4, iota=1)
+    rng = np.random.default_rng(3)
+
+    def batch(k, empty):
+        out = []
+        for m in range(4):
+            ids = []
+            for t, (rows, _, _, _) in enumerate(shape):
+                n = 0 if t in empty else int(rng.integers(0, 700))
+                ids.append(np.minimum(rng.geometric(0.2, n) - 1, rows - 1))
+            out.append(msg(max(0, k - 2 * (m == 2)), ids, dims, 7))
+        return out
+
+    run_custom(cfg, [batch(0, [0, 3]), batch(1, [1, 2, 8]), batch(2, [0, 1, 2, 5, 7, 8]), batch(3, []),
+                     batch(4, [3, 4, 6])])
+
+
+@pytest.mark.parametrize("rule", [None, dict(iota=3, decay=1, lam=0.5), dict(iota=1, row_staleness=1)])
+@pytest.mark.parametrize("tables", [1, 3])
+def test_more_messages_than_the_scan_caches(tables, rule):
+    """A step of so many messages that their lookups stay in global memory,
+    uneven ones (empty, short and long) among them."""
+    M = 1300
+    shape = [(300, 4, 0, 0), (50, 4, 0, 0), (70, 6, 0, 1)][:tables]
+    cfg = cfg_of(shape, D=3, G=M, iota=(rule or {}).get("iota", 1))
+    rng = np.random.default_rng(tables)
+
+    def batch(k):
+        return [msg(max(0, k - int(rng.integers(0, 3))),
+                    [rng.integers(0, s[0], int(rng.integers(0, 4)) + 40 * (m % 97 == 0)) for s in shape],
+                    [s[1] for s in shape], 3) for m in range(M)]
+
+    run_custom(cfg, [batch(0), batch(1)], rule=rule, max_buf=M, max_ids=64)
+
+
 @pytest.mark.parametrize("D", [2048 * 152 * 2 + 6, 2048 * 152 * 3 * 2 + 2048 + 6])
 def test_dense_tiles_over_many_ctas(D):
     """Dense sizes that give some CTAs more tiles than others, a short last
