@@ -20,8 +20,9 @@ using namespace gba;
 namespace {
 
 constexpr int MAX_DIM = 256;
+constexpr int MAX_DIGIT_BITS = 9;  // of a sort pass
+constexpr int MAX_RADIX = 1 << MAX_DIGIT_BITS;
 constexpr int META_SLOTS = 4;
-constexpr int MAX_PASSES = 4;
 constexpr int64_t MAX_STEP_OCC = (1ll << 30) - 1;
 constexpr int MAX_WTAB = 1024;  // decay weights lambda^s for s < MAX_WTAB
 constexpr int EAGER_SLOTS = 8;  // pending global steps with eager dense accumulators
@@ -114,8 +115,7 @@ struct gba_handle {
   gba_staleness_desc st{};
   uint64_t seed = 0;
   int64_t k = 0;
-  uint32_t total_keys_bits = 1;
-  int passes = 1;
+  SortPlan plan{};
 
   std::deque<Msg> fifo;
   bool arenas_ready = false;
@@ -139,7 +139,6 @@ struct gba_handle {
   uint32_t* d_keys[SLOTS][2] = {};
   uint32_t* d_vals[SLOTS][2] = {};
   unsigned long long* d_status[SLOTS] = {};
-  int64_t status_tiles = 0;
   uint32_t epoch = 0;
   char* d_step_scratch[SLOTS] = {};
   StepScratch sc[SLOTS] = {};
@@ -431,8 +430,7 @@ gba_status layout_keys(gba_handle* h) {
   const uint64_t kmax = base > 0 ? base - 1 : 0;
   uint32_t bits = 1;
   while (bits < 32 && (kmax >> bits) != 0) ++bits;
-  h->total_keys_bits = bits;
-  h->passes = (int)((bits + 7) / 8);
+  h->plan = make_sort_plan((int)bits, MAX_DIGIT_BITS);
   if (h->T > 0) {
     GBA_CUDA(h, cudaMemcpy(h->d_tinfo, h->h_tinfo.data(), h->T * sizeof(TableInfo),
                            cudaMemcpyHostToDevice));
@@ -500,7 +498,7 @@ gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
   if (N > h->n_cap) {
     sync_all(h);
     int64_t cap = std::max<int64_t>(N + N / 4, 4096);
-    const int64_t tiles = sort_tiles(cap);
+    const size_t status_bytes = sort_status_words(cap, MAX_RADIX) * sizeof(unsigned long long);
     for (int b = 0; b < SLOTS; ++b) {
       for (int i = 0; i < 2; ++i) {
         cudaFree(h->d_keys[b][i]);
@@ -511,12 +509,10 @@ gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
       }
       cudaFree(h->d_status[b]);
       h->d_status[b] = nullptr;
-      GBA_CUDA(h, cudaMalloc(&h->d_status[b], (size_t)tiles * 256 * sizeof(unsigned long long)));
-      GBA_CUDA(h,
-               cudaMemset(h->d_status[b], 0, (size_t)tiles * 256 * sizeof(unsigned long long)));
+      GBA_CUDA(h, cudaMalloc(&h->d_status[b], status_bytes));
+      GBA_CUDA(h, cudaMemset(h->d_status[b], 0, status_bytes));
     }
     h->n_cap = cap;
-    h->status_tiles = tiles;
     // row-kernel buffers: a record per possible row (and one for the totals),
     // a kept-list entry per occurrence, look-back words per scan tile,
     // long rows and their chunks
@@ -904,7 +900,7 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
   }
   {
     const size_t M = (size_t)max_buffered_msgs;
-    const size_t bytes = align16(MAX_PASSES * 256 * 4) + align16(MAX_PASSES * 4) +
+    const size_t bytes = align16(MAX_PASSES * MAX_RADIX * 4) + align16(MAX_PASSES * 4) +
                          align16(M * 4) + align16(M * 4) + align16(4) + align16(4) +
                          align16((size_t)std::max(h->T, 1) * 32) + align16(M * 4);
     for (int b = 0; b < SLOTS; ++b) {
@@ -913,7 +909,7 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
       char* p = h->d_step_scratch[b];
       StepScratch& sc = h->sc[b];
       sc.hist = (uint32_t*)p;
-      p += align16(MAX_PASSES * 256 * 4);
+      p += align16(MAX_PASSES * MAX_RADIX * 4);
       sc.tile_counter = (uint32_t*)p;
       p += align16(MAX_PASSES * 4);
       sc.keep = (int32_t*)p;
@@ -1124,7 +1120,7 @@ int32_t gba_try_apply(gba_handle* h) {
   // ---- K1: message weights (Eq. (1)); clears the per-step scratch
   {
     Timed tm(h, GBA_K_WEIGHTS, h->sorts);
-    launch_weights(a, sc, h->d_stats, MAX_PASSES * 256, h->sorts);
+    launch_weights(a, sc, h->d_stats, MAX_PASSES * MAX_RADIX, h->sorts);
   }
   // ---- K5 on the side stream, concurrently with the sort and segment-sum.
   // It is forked after the histogram kernel has validated every id, so a step
@@ -1159,19 +1155,27 @@ int32_t gba_try_apply(gba_handle* h) {
   if (N > 0) {
     {
       Timed tm(h, GBA_K_SORT_HIST, h->sorts);
-      int grid = (int)std::min<int64_t>((N + 255) / 256, (int64_t)h->num_sms * 8);
       // the first pass writes buffer 0, so its input keys go to buffer 1
-      launch_sort_histogram(a, h->passes, sc, h->d_keys[b][1], sink, std::max(grid, 1), h->sorts);
+      launch_sort_histogram(a, h->plan, sc.hist, h->d_keys[b][1], sink, h->num_sms, h->sorts);
     }
     launch_dense_side();
     const uint32_t* kin = h->d_keys[b][1];
     const uint32_t* vin = nullptr;
-    for (int p = 0; p < h->passes; ++p) {
+    for (int p = 0; p < h->plan.passes; ++p) {
       const int ob = p & 1;
       if (++h->epoch == 0u) h->epoch = 1u;
       Timed tm(h, GBA_K_SORT_PASS, h->sorts);
-      launch_onesweep(a, p == 0, p, kin, vin, h->d_keys[b][ob], h->d_vals[b][ob], sc,
-                      h->d_status[b], h->epoch, sink, h->wait_ns, h->sorts);
+      SortPass sp{};
+      sp.N = (uint32_t)N;
+      sp.hist = sc.hist + p * h->plan.radix;
+      sp.ticket = sc.tile_counter + p;
+      sp.keys_in = kin;
+      sp.vals_in = vin;
+      sp.keys_out = h->d_keys[b][ob];
+      sp.vals_out = h->d_vals[b][ob];
+      sp.status = h->d_status[b];
+      sp.epoch = h->epoch;
+      launch_onesweep(h->plan, p, sp, sink, h->wait_ns, h->sorts);
       kin = h->d_keys[b][ob];
       vin = h->d_vals[b][ob];
       final_buf = ob;

@@ -282,7 +282,7 @@ struct StepArgs {
 
 // Per-step device scratch that K1 clears at the start of a step.
 struct StepScratch {
-  uint32_t* hist;          // [4][256] digit histograms of the key passes
+  uint32_t* hist;          // [passes][radix] digit histograms of the key passes
   uint32_t* tile_counter;  // [4] onesweep tile tickets
   int32_t* keep;           // [M] message weights f
   int32_t* kept_list;      // [M] indices of kept messages, in pop order
@@ -331,14 +331,13 @@ struct DevStats {
       occ_kept;
 };
 
-// The message that holds table-local occurrence x: the largest m in [0, M)
-// with off[m] <= x, given off[0] = 0 <= x < off[M] (empty messages repeat an
-// offset and are skipped by taking the largest such m).
-__device__ __forceinline__ int message_of(const uint32_t* off, int M, uint32_t x) {
-  int lo = 0, hi = M;  // off[lo] <= x < off[hi]
+// The message of table-local occurrence x in the offsets off[0..M]: the
+// largest m with off[m] <= x (empty messages repeat an offset).
+__device__ __forceinline__ int message_of_any(const uint32_t* off, int M, uint32_t x) {
+  int lo = 0, hi = M;
   while (hi - lo > 1) {
-    int mid = (lo + hi) >> 1;
-    if (__ldg(off + mid) <= x)
+    const int mid = (lo + hi) >> 1;
+    if (off[mid] <= x)
       lo = mid;
     else
       hi = mid;
@@ -346,27 +345,73 @@ __device__ __forceinline__ int message_of(const uint32_t* off, int M, uint32_t x
   return lo;
 }
 
+// The same, starting from the message an even split would give (exact when
+// every message holds the same number of ids, as with one-hot fields; scale
+// is M over the table's occurrences), then a few neighbours, then the binary
+// search.  x becomes the occurrence's index within its message.
+__device__ __forceinline__ int message_of(const uint32_t* off, int M, uint32_t& x, float scale) {
+  int m = min((int)((float)x * scale), M - 1);
+  uint32_t lo = off[m], hi = off[m + 1];
+  if (x < lo || x >= hi) {
+    for (int s = 0; s < 3 && (x < lo || x >= hi); ++s) {
+      if (x < lo) {
+        hi = lo;
+        lo = off[--m];  // off[0] = 0 <= x: m stays >= 0
+      } else {
+        lo = hi;
+        hi = off[++m + 1];  // x < off[M]: m stays < M
+      }
+    }
+    if (x < lo || x >= hi) {
+      m = message_of_any(off, M, x);
+      lo = off[m];
+    }
+  }
+  x -= lo;
+  return m;
+}
+
 // ---- launch wrappers (defined in the kernel translation units) ---------------
 void launch_weights(const StepArgs& a, StepScratch sc, DevStats* stats, int n_hist_words,
                     cudaStream_t s);
 
-// Keys per onesweep tile (also sizes the look-back words of the static sort).
-#ifndef GBA_SORT_TILE
-#define GBA_SORT_TILE 2048
-#endif
-constexpr int SORT_TILE_KEYS = GBA_SORT_TILE;  // keys per onesweep tile
+// ---- the sort of the step's keys
+constexpr int MAX_PASSES = 4;
+// Keys per onesweep tile, and of more than SORT_BIG_N keys twice as many.
+constexpr int SORT_TILE_KEYS = 2048;
+constexpr int64_t SORT_BIG_N = 1 << 21;
 
-// Digit histograms of every pass; writes each occurrence's key to keys0 (the
-// first onesweep pass's input).
-void launch_sort_histogram(const StepArgs& a, int passes, StepScratch sc, uint32_t* keys0,
-                           ErrSink err, int grid, cudaStream_t s);
+// The digits of the passes over keys of so many bits.
+struct SortPlan {
+  int32_t passes;
+  int32_t radix;  // counters per pass: 256 or 512
+  int32_t shift[MAX_PASSES];
+  uint32_t mask[MAX_PASSES];
+};
+SortPlan make_sort_plan(int key_bits, int max_digit_bits);
+// Look-back words for sorts of up to N keys.
+size_t sort_status_words(int64_t N, int radix);
 
-void launch_onesweep(const StepArgs& a, bool first, int pass, const uint32_t* keys_in,
-                     const uint32_t* vals_in, uint32_t* keys_out, uint32_t* vals_out,
-                     StepScratch sc, unsigned long long* status, uint32_t epoch, ErrSink err,
-                     int64_t wait_ns, cudaStream_t s);
+// Digit counts of every pass into hist [passes][radix]; writes each
+// occurrence's key to keys0 (the first pass's input).
+void launch_sort_histogram(const StepArgs& a, const SortPlan& plan, uint32_t* hist,
+                           uint32_t* keys0, ErrSink err, int num_sms, cudaStream_t s);
 
-int sort_tiles(int64_t N);
+struct SortPass {
+  uint32_t N;
+  int32_t shift;  // set by launch_onesweep, as is mask
+  uint32_t mask;
+  const uint32_t* hist;  // the pass's digit counts
+  uint32_t* ticket;
+  const uint32_t* keys_in;
+  const uint32_t* vals_in;  // unused by the first pass: its payload is the position
+  uint32_t* keys_out;
+  uint32_t* vals_out;
+  unsigned long long* status;
+  uint32_t epoch;
+};
+void launch_onesweep(const SortPlan& plan, int pass, SortPass sp, ErrSink err, int64_t wait_ns,
+                     cudaStream_t s);
 
 // One table as the row kernels see it.
 struct SegTable {

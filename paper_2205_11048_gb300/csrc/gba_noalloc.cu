@@ -47,11 +47,8 @@ constexpr size_t kOffTinfo = kOffNbase + 16;
 constexpr size_t kOffErr = kOffTinfo + 32;  // TableInfo is 24 bytes
 static_assert(sizeof(gba::TableInfo) <= 32, "TableInfo outgrew its scratch slot");
 constexpr size_t kBytes = kOffErr + 16;
-#if GBA_SORT_TILE == 2048
 static_assert(kBytes == GBA_STATIC_SORT_BYTES, "scratch size differs from the header");
-#else
-static_assert(kBytes <= GBA_STATIC_SORT_BYTES, "scratch larger than the header's size");
-#endif
+static_assert(kMaxIds <= SORT_BIG_N, "the look-back words are sized for the smaller tiles");
 
 static __device__ __align__(256) unsigned char g_sort_scratch[kBytes];
 
@@ -138,19 +135,17 @@ extern "C" gba_status gba_sort_ids_static(const int64_t* ids, int64_t n, int64_t
   a.ids_ptr = reinterpret_cast<const int64_t* const*>(base + kOffIdsPtr);
   a.nbase = reinterpret_cast<const int64_t*>(base + kOffNbase);
   a.tinfo = reinterpret_cast<const TableInfo*>(base + kOffTinfo);
-  StepScratch sc{};
-  sc.hist = reinterpret_cast<uint32_t*>(base + kOffHist);
-  sc.tile_counter = reinterpret_cast<uint32_t*>(base + kOffTiles);
+  uint32_t* hist = reinterpret_cast<uint32_t*>(base + kOffHist);
+  uint32_t* tickets = reinterpret_cast<uint32_t*>(base + kOffTiles);
   uint32_t* err_words = reinterpret_cast<uint32_t*>(base + kOffErr);
   ErrSink err{err_words, err_words, err_words + 1};
 
   uint64_t kmax = (uint64_t)rows - 1;
   int bits = 1;
   while (bits < 32 && (kmax >> bits) != 0) ++bits;
-  const int passes = (bits + 7) / 8;
+  const SortPlan plan = make_sort_plan(bits, 8);  // the scratch holds 256 counters per pass
+  const int passes = plan.passes;
 
-  int grid = (int)((n + 255) / 256);
-  if (grid > 152 * 8) grid = 152 * 8;
   // Ping-pong between the scratch pair and the caller's outputs so that the
   // last pass lands in the outputs; the first pass reads the keys the
   // histogram kernel wrote into the buffer that pass does not write.
@@ -158,7 +153,7 @@ extern "C" gba_status gba_sort_ids_static(const int64_t* ids, int64_t n, int64_t
   uint32_t* tmp_v = reinterpret_cast<uint32_t*>(base + kOffVals);
   unsigned long long* status = reinterpret_cast<unsigned long long*>(base + kOffStatus);
   uint32_t* keys0 = ((passes - 1) % 2) == 0 ? tmp_k : rows_out;
-  launch_sort_histogram(a, passes, sc, keys0, err, grid, s);
+  launch_sort_histogram(a, plan, hist, keys0, err, 152, s);
   const uint32_t* kin = keys0;
   const uint32_t* vin = nullptr;
   for (int p = 0; p < passes; ++p) {
@@ -167,7 +162,17 @@ extern "C" gba_status gba_sort_ids_static(const int64_t* ids, int64_t n, int64_t
     uint32_t* vo = to_out ? order_out : tmp_v;
     uint32_t ep = g_epoch[dev].fetch_add(1u) + 1u;
     if (ep == 0u) ep = g_epoch[dev].fetch_add(1u) + 1u;
-    launch_onesweep(a, p == 0, p, kin, vin, ko, vo, sc, status, ep, err, 2000000000ll, s);
+    SortPass sp{};
+    sp.N = (uint32_t)n;
+    sp.hist = hist + p * plan.radix;
+    sp.ticket = tickets + p;
+    sp.keys_in = kin;
+    sp.vals_in = vin;
+    sp.keys_out = ko;
+    sp.vals_out = vo;
+    sp.status = status;
+    sp.epoch = ep;
+    launch_onesweep(plan, p, sp, err, 2000000000ll, s);
     kin = ko;
     vin = vo;
   }

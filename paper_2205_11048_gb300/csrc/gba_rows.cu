@@ -80,46 +80,6 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
-// The message of table-local occurrence x in the offsets off[0..M]: the
-// largest m with off[m] <= x (empty messages repeat an offset).
-__device__ __forceinline__ int message_of_any(const uint32_t* off, int M, uint32_t x) {
-  int lo = 0, hi = M;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (off[mid] <= x)
-      lo = mid;
-    else
-      hi = mid;
-  }
-  return lo;
-}
-
-// The same, starting from the message an even split would give (exact when
-// every message holds the same number of ids, as with one-hot fields; scale
-// is M over the table's occurrences), then a few neighbours, then the binary
-// search.  x becomes the occurrence's index within its message.
-__device__ __forceinline__ int message_of(const uint32_t* off, int M, uint32_t& x, float scale) {
-  int m = min((int)((float)x * scale), M - 1);
-  uint32_t lo = off[m], hi = off[m + 1];
-  if (x < lo || x >= hi) {
-    for (int s = 0; s < 3 && (x < lo || x >= hi); ++s) {
-      if (x < lo) {
-        hi = lo;
-        lo = off[--m];  // off[0] = 0 <= x: m stays >= 0
-      } else {
-        lo = hi;
-        hi = off[++m + 1];  // x < off[M]: m stays < M
-      }
-    }
-    if (x < lo || x >= hi) {
-      m = message_of_any(off, M, x);
-      lo = off[m];
-    }
-  }
-  x -= lo;
-  return m;
-}
-
 __device__ __forceinline__ int32_t token32(int64_t token) {  // tags stay below 2^31
   return token > 0x7FFFFFFFll ? 0x7FFFFFFF : (int32_t)token;
 }

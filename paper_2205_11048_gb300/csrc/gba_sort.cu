@@ -2,41 +2,26 @@
 // row keys) of the GBA aggregate-and-apply step.
 //
 // The sort follows the onesweep method (Adinets & Merrill 2022): one kernel
-// counts the digits of every pass, then each pass is a single kernel in which
-// tiles rank their keys locally and find their global output offsets by
-// decoupled look-back over the per-tile digit counts of earlier tiles
-// (Merrill & Garland 2016).  Tiles take tickets from an atomic counter, so a
-// tile only ever waits on tiles that are already running; every wait is
-// bounded in time and latches ERR_TIMEOUT instead of hanging.
-//
-// The first pass reads the int64 ids straight from the messages and computes
-// the 32-bit key (global row = table key base + row) on the fly, with the
-// global occurrence index as payload; later passes move (key, payload) pairs.
+// maps the ids to 32-bit keys (global row = table key base + row) and counts
+// the digits of every pass, then each pass is a single kernel in which tiles
+// rank their keys locally and find their global output offsets by decoupled
+// look-back over the per-tile digit counts of earlier tiles (Merrill & Garland
+// 2016).  Tiles take tickets from an atomic counter, so a tile only ever waits
+// on tiles that are already running; every wait is bounded in time and latches
+// ERR_TIMEOUT instead of hanging.  The payload is the global occurrence index.
+#include <algorithm>
+
 #include "gba_internal.cuh"
 
 namespace gba {
 
 namespace {
 
-constexpr int RADIX = 256;
-constexpr int SORT_THREADS = 256;  // one thread per digit in the look-back
+constexpr int SORT_THREADS = 256;
 constexpr int SORT_WARPS = SORT_THREADS / 32;
-constexpr int SORT_ITEMS = SORT_TILE_KEYS / SORT_THREADS;
-constexpr int SORT_TILE = SORT_TILE_KEYS;
-static_assert(SORT_TILE_KEYS % SORT_THREADS == 0, "tile must fill the block");
-constexpr int MAX_PASSES = 4;
-constexpr int LB_WIN = 8;  // look-back window
 constexpr int OFF_CACHE = 1024;  // message offsets kept in shared memory
-
-// Copies the step's message offsets into shared memory when they fit;
-// returns the array the key computation should read.
-__device__ __forceinline__ const uint32_t* cache_offsets(const StepArgs& a, uint32_t* s_off) {
-  const int n = a.T * (a.M + 1);
-  if (n > OFF_CACHE) return a.msg_off;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s_off[i] = a.msg_off[i];
-  __syncthreads();
-  return s_off;
-}
+constexpr int TAB_CACHE = 64;    // tables whose bounds are kept in shared memory
+constexpr uint32_t FULL = 0xffffffffu;
 
 // Look-back status word: [63:32] epoch of the launch, [31:30] flag, [29:0] count.
 constexpr unsigned long long FLAG_AGG = 1ull << 30;
@@ -61,35 +46,16 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
-// Key of global occurrence o: the table holding o, the message holding it, the
-// id, and the row it maps to (DIRECT ids outside [0, V) latch ERR_ID_RANGE and
+// Row of an id in table t (DIRECT ids outside [0, V) latch ERR_ID_RANGE and
 // are clamped to row 0; the whole step is then skipped by later kernels).
-__device__ __forceinline__ uint32_t occurrence_key(const StepArgs& a, const uint32_t* offs,
-                                                   int64_t o, const ErrSink& err) {
-  int t = 0;
-  while (t + 1 < a.T && __ldg(a.nbase + t + 1) <= o) ++t;
-  const uint32_t ot = (uint32_t)(o - __ldg(a.nbase + t));
-  const uint32_t* off = offs + (size_t)t * (a.M + 1);
-  int lo = 0, hi = a.M;  // the message holding ot: off[lo] <= ot < off[lo + 1]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (off[mid] <= ot)
-      lo = mid;
-    else
-      hi = mid;
-  }
-  const int m = lo;
-  const uint32_t p = ot - off[m];
-  const int64_t* ids = a.ids_ptr[(size_t)t * a.M + m];
-  const int64_t id = __ldg(ids + p);
-  const TableInfo ti = a.tinfo[t];
+__device__ __forceinline__ uint64_t row_of_id(const StepArgs& a, const TableInfo& ti, int t,
+                                              int64_t id, const ErrSink& err) {
   uint64_t row;
   if (ti.id_mode == 0) {
+    row = (uint64_t)id;
     if (id < 0 || id >= ti.V) {
       raise_error(err, ERR_ID_RANGE);
       row = 0;
-    } else {
-      row = (uint64_t)id;
     }
   } else if (ti.id_mode == 1) {
     row = mod_u64((uint64_t)id, (uint64_t)ti.V, ti.mod_magic);
@@ -105,26 +71,7 @@ __device__ __forceinline__ uint32_t occurrence_key(const StepArgs& a, const uint
       }
     }
   }
-  return ti.key_base + (uint32_t)row;
-}
-
-// Exclusive scan of one value per thread over a 256-thread block.
-__device__ __forceinline__ uint32_t block_excl_scan_256(uint32_t v, uint32_t* s_tmp) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) s_tmp[warp] = x;
-  __syncthreads();
-  uint32_t wsum = 0;
-#pragma unroll
-  for (int w = 0; w < SORT_WARPS; ++w)
-    if (w < warp) wsum += s_tmp[w];
-  __syncthreads();
-  return wsum + x - v;
+  return row;
 }
 
 // ---------------------------------------------------------------------------
@@ -184,48 +131,105 @@ __global__ void __launch_bounds__(256) k_message_weights(StepArgs a, StepScratch
 }
 
 // ---------------------------------------------------------------------------
-// Digit counts of every pass in one read of the ids; also writes every
-// occurrence's key (keys0) for the first onesweep pass.
+// Keys of every occurrence (keys0, the first pass's input) and the digit counts
+// of every pass, in one read of the ids.
+//
+// Latency of the id gathers and, on small steps, the merging of the blocks'
+// counts bound this kernel: four ids are in flight per thread, and a block takes
+// 2,048 keys (1,024 while there are fewer blocks than two per SM) before it adds
+// its counts to the step's.  0.85M ids 17 -> 11.5 us, 131M 959 -> 719.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(SORT_THREADS) k_sort_histogram(StepArgs a, int passes,
-                                                                 StepScratch sc, uint32_t* keys0,
-                                                                 ErrSink err) {
+constexpr int HIST_ITEMS = 4;  // ids in flight per thread
+
+template <int RADIX>
+__global__ void __launch_bounds__(SORT_THREADS)
+    k_sort_histogram(StepArgs a, SortPlan plan, uint32_t* __restrict__ hist,
+                     uint32_t* __restrict__ keys0, ErrSink err) {
   __shared__ uint32_t h[MAX_PASSES][RADIX];
   __shared__ uint32_t s_off[OFF_CACHE];
-  for (int i = threadIdx.x; i < MAX_PASSES * RADIX; i += SORT_THREADS) (&h[0][0])[i] = 0u;
-  const uint32_t* offs = cache_offsets(a, s_off);
+  __shared__ uint32_t s_nb[TAB_CACHE + 1];
+  const int tid = threadIdx.x;
+  for (int i = tid; i < MAX_PASSES * RADIX; i += SORT_THREADS) (&h[0][0])[i] = 0u;
+  const int T = a.T, M = a.M;
+  const bool offs_cached = T * (M + 1) <= OFF_CACHE, tabs_cached = T <= TAB_CACHE;
+  if (offs_cached)
+    for (int i = tid; i < T * (M + 1); i += SORT_THREADS) s_off[i] = a.msg_off[i];
+  if (tabs_cached)
+    for (int i = tid; i <= T; i += SORT_THREADS) s_nb[i] = (uint32_t)a.nbase[i];
   __syncthreads();
-  const int64_t stride = (int64_t)gridDim.x * SORT_THREADS;
-  for (int64_t o = (int64_t)blockIdx.x * SORT_THREADS + threadIdx.x; o < a.N; o += stride) {
-    const uint32_t key = occurrence_key(a, offs, o, err);
-    keys0[o] = key;
-    for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(key >> (8 * p)) & (RADIX - 1)], 1u);
+  const uint32_t* offs = offs_cached ? s_off : a.msg_off;
+  const uint32_t N = (uint32_t)a.N;  // below 2^30
+  auto first_of = [&](int t) { return tabs_cached ? s_nb[t] : (uint32_t)__ldg(a.nbase + t); };
+  const uint32_t step = (uint32_t)(SORT_THREADS * HIST_ITEMS);
+  for (uint32_t base = blockIdx.x * step; base < N; base += gridDim.x * step) {
+    int64_t id[HIST_ITEMS];
+    int tab[HIST_ITEMS];
+#pragma unroll
+    for (int e = 0; e < HIST_ITEMS; ++e) {
+      const uint32_t o = base + (uint32_t)(e * SORT_THREADS + tid);
+      tab[e] = -1;
+      if (o >= N) continue;
+      int lo = 0, hi = T;  // the last table that starts at or before o
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (first_of(mid) <= o)
+          lo = mid;
+        else
+          hi = mid;
+      }
+      const uint32_t nb = first_of(lo), n = first_of(lo + 1) - nb;
+      uint32_t x = o - nb;
+      const int m = message_of(offs + (size_t)lo * (M + 1), M, x, __fdividef((float)M, (float)n));
+      tab[e] = lo;
+      id[e] = __ldg(a.ids_ptr[(size_t)lo * M + m] + x);
+    }
+#pragma unroll
+    for (int e = 0; e < HIST_ITEMS; ++e) {
+      if (tab[e] < 0) continue;
+      const TableInfo ti = a.tinfo[tab[e]];
+      const uint32_t key = ti.key_base + (uint32_t)row_of_id(a, ti, tab[e], id[e], err);
+      keys0[base + (uint32_t)(e * SORT_THREADS + tid)] = key;
+#pragma unroll
+      for (int p = 0; p < MAX_PASSES; ++p)
+        if (p < plan.passes) atomicAdd(&h[p][(key >> plan.shift[p]) & plan.mask[p]], 1u);
+    }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < passes * RADIX; i += SORT_THREADS) {
+  for (int i = tid; i < plan.passes * RADIX; i += SORT_THREADS) {
     const uint32_t v = (&h[0][0])[i];
-    if (v) atomicAdd(sc.hist + i, v);
+    if (v) atomicAdd(hist + i, v);
   }
 }
 
 // ---------------------------------------------------------------------------
-// One onesweep pass over 8 bits of the key.
+// One onesweep pass.
+//
+// Bound by instruction issue and latency: 16 B move per key, and a key costs
+// about four warp instructions of 32.  Keys and payloads go to shared memory in
+// digit order before the look-back, so that few registers live through it (48
+// instead of 80: five blocks per SM instead of three); a short last tile is
+// padded with the largest key, which needs no checks; match.any groups equal
+// digits (ballots per bit: 1.12 ms a pass against 0.83 on 131M keys).  Above
+// SORT_BIG_N keys a tile holds 4,096 of them (5.2M keys: 70 us a pass against 89
+// with 2,048).  Digits are 8 bits wide, or up to 9 where that saves a pass: 26-bit
+// keys take three passes.  131M keys: 4 x 1.46 -> 1.12 + 2 x 0.83 ms.
 // ---------------------------------------------------------------------------
 #ifndef GBA_LOOKBACK_SLEEP_NS
 #define GBA_LOOKBACK_SLEEP_NS 64
 #endif
-template <bool FIRST>
-__global__ void __launch_bounds__(SORT_THREADS)
-    k_onesweep(StepArgs a, int pass, const uint32_t* __restrict__ keys_in,
-               const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
-               uint32_t* __restrict__ vals_out, StepScratch sc, unsigned long long* status,
-               uint32_t epoch, ErrSink err, int64_t wait_ns) {
-  __shared__ uint32_t s_warp[SORT_WARPS][RADIX];  // per-warp digit counts, then offsets
-  __shared__ uint32_t s_tile_excl[RADIX];         // first tile slot of each digit
-  __shared__ uint32_t s_out_base[RADIX];          // global position of that slot
-  __shared__ uint32_t s_tmp[SORT_WARPS];
-  __shared__ uint32_t s_keys[SORT_TILE];
-  __shared__ uint32_t s_vals[SORT_TILE];
+template <int ITEMS, int RADIX, bool FIRST>
+__global__ void __launch_bounds__(SORT_THREADS, ITEMS == 8 ? 5 : 4)
+    k_onesweep(SortPass sp, ErrSink err, int64_t wait_ns) {
+  constexpr int TILE = ITEMS * SORT_THREADS;
+  constexpr int DPT = RADIX / SORT_THREADS;  // digits per thread: tid * DPT ..
+  constexpr int WIN = DPT == 1 ? 8 : 4;      // look-back window
+  static_assert(DPT == 1 || DPT == 2, "one or two digits per thread");
+  __shared__ __align__(4) uint16_t s_cnt[SORT_WARPS][RADIX];  // per-warp digit counts, then offsets
+  __shared__ uint32_t s_excl[RADIX];  // first tile slot of each digit
+  __shared__ uint32_t s_out[RADIX];   // output position of tile slot 0 of each digit
+  __shared__ uint32_t s_tmp[2][SORT_WARPS];
+  __shared__ uint32_t s_keys[TILE];
+  __shared__ uint32_t s_vals[TILE];
   __shared__ uint32_t s_tile;
 
   // An id range error was latched before this launch (by the histogram):
@@ -233,92 +237,165 @@ __global__ void __launch_bounds__(SORT_THREADS)
   if (__syncthreads_or((ld_volatile_u32(err.step) & ERR_ID_RANGE) != 0u)) return;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_tile = atomicAdd(sc.tile_counter + pass, 1u);
-  for (int i = tid; i < SORT_WARPS * RADIX; i += SORT_THREADS) (&s_warp[0][0])[i] = 0u;
+  if (tid == 0) s_tile = atomicAdd(sp.ticket, 1u);
+  uint32_t* cnt_words = reinterpret_cast<uint32_t*>(&s_cnt[0][0]);
+  for (int i = tid; i < SORT_WARPS * RADIX / 2; i += SORT_THREADS) cnt_words[i] = 0u;
+  uint32_t hist_d[DPT];
+#pragma unroll
+  for (int q = 0; q < DPT; ++q) hist_d[q] = sp.hist[tid * DPT + q];
   __syncthreads();
 
-  const uint32_t tile = s_tile;
-  const int64_t N = a.N;
-  const int64_t base = (int64_t)tile * SORT_TILE;
-  const int shift = 8 * pass;
+  const uint32_t tile = s_tile, N = sp.N;
+  const uint32_t base = tile * (uint32_t)TILE;
+  const uint32_t n_valid = min(N - base, (uint32_t)TILE);
+  const int shift = sp.shift;
+  const uint32_t mask = sp.mask;
 
-  uint32_t key[SORT_ITEMS], val[SORT_ITEMS], rank[SORT_ITEMS];
+  // The slots past the end hold the largest key: they are the last of the last
+  // digit, so they rank behind every key and are taken off that digit's count.
+  uint32_t key[ITEMS], val[ITEMS];
+  const uint32_t at = (uint32_t)(warp * (ITEMS * 32) + lane);
+  if (n_valid == (uint32_t)TILE) {
 #pragma unroll
-  for (int j = 0; j < SORT_ITEMS; ++j) {
-    const int64_t idx = base + (int64_t)warp * (SORT_ITEMS * 32) + j * 32 + lane;
-    if (idx < N) {
-      if (FIRST) {  // keys written by the histogram kernel; payload = occurrence
-        key[j] = keys_in[idx];
-        val[j] = (uint32_t)idx;
-      } else {
-        key[j] = keys_in[idx];
-        val[j] = vals_in[idx];
-      }
-    } else {
-      key[j] = 0u;
-      val[j] = 0u;
+    for (int j = 0; j < ITEMS; ++j) {
+      key[j] = sp.keys_in[base + at + j * 32];
+      val[j] = FIRST ? base + at + j * 32 : sp.vals_in[base + at + j * 32];
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      const bool in = at + j * 32 < n_valid;
+      key[j] = in ? sp.keys_in[base + at + j * 32] : 0xFFFFFFFFu;
+      val[j] = FIRST ? base + at + j * 32 : (in ? sp.vals_in[base + at + j * 32] : 0u);
     }
   }
 
   // Warp-level multi-split: stable rank of each key among equal digits.
   const uint32_t lt = lanemask_lt();
+  uint32_t rank[ITEMS / 2];  // two 16-bit ranks each
 #pragma unroll
-  for (int j = 0; j < SORT_ITEMS; ++j) {
-    const int64_t idx = base + (int64_t)warp * (SORT_ITEMS * 32) + j * 32 + lane;
-    const bool valid = idx < N;
-    const uint32_t d = valid ? ((key[j] >> shift) & (RADIX - 1)) : (uint32_t)RADIX;
-    const uint32_t peers = __match_any_sync(0xffffffffu, d);
-    uint32_t before = 0;
-    if (valid) before = s_warp[warp][d];
-    rank[j] = before + __popc(peers & lt);
+  for (int j = 0; j < ITEMS; ++j) {
+    const uint32_t d = (key[j] >> shift) & mask;
+    const uint32_t peers = __match_any_sync(FULL, d);
+    const uint32_t before = s_cnt[warp][d];
+    const uint32_t r = before + __popc(peers & lt);
+    rank[j / 2] = (j & 1) ? rank[j / 2] | (r << 16) : r;
     __syncwarp();
-    if (valid && (peers & lt) == 0u) s_warp[warp][d] = before + __popc(peers);
+    if ((peers & lt) == 0u) s_cnt[warp][d] = (uint16_t)(before + __popc(peers));
     __syncwarp();
   }
   __syncthreads();
 
-  // Thread d: this tile's count of digit d, then its global offset.
-  const int d = tid;
-  uint32_t run = 0;
+  // This thread's digits: the warps' offsets, the tile's counts, published for
+  // the tiles that follow.
+  uint32_t count[DPT];
+  if constexpr (DPT == 1) {
+    uint32_t run = 0u;
 #pragma unroll
-  for (int w = 0; w < SORT_WARPS; ++w) {
-    const uint32_t c = s_warp[w][d];
-    s_warp[w][d] = run;
-    run += c;
+    for (int w = 0; w < SORT_WARPS; ++w) {
+      const uint32_t c = s_cnt[w][tid];
+      s_cnt[w][tid] = (uint16_t)run;
+      run += c;
+    }
+    count[0] = run;
+  } else {  // both digits in one word: a count is at most TILE < 2^16
+    uint32_t run = 0u;
+#pragma unroll
+    for (int w = 0; w < SORT_WARPS; ++w) {
+      uint32_t* word = reinterpret_cast<uint32_t*>(&s_cnt[w][2 * tid]);
+      const uint32_t c = *word;
+      *word = run;
+      run += c;
+    }
+    count[0] = run & 0xFFFFu;
+    count[DPT - 1] = run >> 16;
   }
-  const uint32_t tile_count = run;
-  unsigned long long* my = status + (size_t)tile * RADIX + d;
-  const unsigned long long ep = (unsigned long long)epoch << 32;
-  st_relaxed_u64(my, ep | (tile == 0 ? FLAG_INCL : FLAG_AGG) | tile_count);
+#pragma unroll
+  for (int q = 0; q < DPT; ++q)
+    if ((uint32_t)(tid * DPT + q) == mask) count[q] -= (uint32_t)TILE - n_valid;
+  unsigned long long* my = sp.status + (size_t)tile * RADIX + tid * DPT;
+  const unsigned long long ep = (unsigned long long)sp.epoch << 32;
+#pragma unroll
+  for (int q = 0; q < DPT; ++q)
+    st_relaxed_u64(my + q, ep | (tile == 0 ? FLAG_INCL : FLAG_AGG) | count[q]);
 
-  const uint32_t g_excl = block_excl_scan_256(sc.hist[pass * RADIX + d], s_tmp);
-  const uint32_t t_excl = block_excl_scan_256(tile_count, s_tmp);
-  s_tile_excl[d] = t_excl;
+  // Exclusive scans over the digits of the tile's counts and of the step's.
+  uint32_t t_sum = 0u, g_sum = 0u;
+#pragma unroll
+  for (int q = 0; q < DPT; ++q) {
+    t_sum += count[q];
+    g_sum += hist_d[q];
+  }
+  uint32_t t_inc = t_sum, g_inc = g_sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(FULL, t_inc, o), z = __shfl_up_sync(FULL, g_inc, o);
+    if (lane >= o) {
+      t_inc += y;
+      g_inc += z;
+    }
+  }
+  if (lane == 31) {
+    s_tmp[0][warp] = t_inc;
+    s_tmp[1][warp] = g_inc;
+  }
+  __syncthreads();
+  uint32_t t_excl = t_inc - t_sum, g_excl = g_inc - g_sum;
+#pragma unroll
+  for (int w = 0; w < SORT_WARPS; ++w)
+    if (w < warp) {
+      t_excl += s_tmp[0][w];
+      g_excl += s_tmp[1][w];
+    }
+  s_excl[tid * DPT] = t_excl;
+  if constexpr (DPT == 2) s_excl[tid * DPT + 1] = t_excl + count[0];
+  __syncthreads();
 
-  // Decoupled look-back over a window of LB_WIN predecessors at a time: the
+  // Keys and payloads in digit order in shared memory.
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    const uint32_t d = (key[j] >> shift) & mask;
+    const uint32_t r = (j & 1) ? rank[j / 2] >> 16 : rank[j / 2] & 0xFFFFu;
+    const uint32_t pos = s_excl[d] + s_cnt[warp][d] + r;
+    s_keys[pos] = key[j];
+    s_vals[pos] = val[j];
+  }
+
+  // Decoupled look-back over a window of WIN predecessors at a time: the
   // window's status words are read with independent loads, then consumed from
   // the nearest tile backwards until an inclusive prefix is found.  The words
   // are self-contained (no other data is published with them), so relaxed
   // loads and stores suffice.
-  uint32_t prefix = 0;
+  uint32_t prefix[DPT];
+#pragma unroll
+  for (int q = 0; q < DPT; ++q) prefix[q] = 0u;
   if (tile > 0) {
-    int64_t j = (int64_t)tile - 1;
+    int j = (int)tile - 1;
     const uint64_t t0 = globaltimer_ns();
     bool done = false;
     while (!done) {
-      unsigned long long v[LB_WIN];
+      unsigned long long v[WIN][DPT];
 #pragma unroll
-      for (int i = 0; i < LB_WIN; ++i)
-        v[i] = (j - i >= 0) ? ld_relaxed_u64(status + (size_t)(j - i) * RADIX + d) : 0ull;
+      for (int i = 0; i < WIN; ++i)
+#pragma unroll
+        for (int q = 0; q < DPT; ++q)
+          v[i][q] = j - i >= 0
+                        ? ld_relaxed_u64(sp.status + (size_t)(j - i) * RADIX + tid * DPT + q)
+                        : 0ull;
       int used = 0;
 #pragma unroll
-      for (int i = 0; i < LB_WIN; ++i) {
-        if (done || used != i || j - i < 0) continue;
-        const unsigned long long x = v[i];
-        if ((x & ~0xFFFFFFFFull) != ep || (x & FLAG_MASK) == 0ull) continue;  // not ready
-        prefix += (uint32_t)(x & COUNT_MASK);
+      for (int i = 0; i < WIN; ++i) {
+        if (done || used != i) continue;
+        // ready once the words carry this launch's epoch and one flag (before
+        // tile 0 there are none: zero words are never ready)
+        const unsigned long long tag = v[i][0] & ~COUNT_MASK;
+        if ((tag >> 32) != (ep >> 32) || (tag & FLAG_MASK) == 0ull ||
+            (v[i][DPT - 1] & ~COUNT_MASK) != tag)
+          continue;
+#pragma unroll
+        for (int q = 0; q < DPT; ++q) prefix[q] += (uint32_t)(v[i][q] & COUNT_MASK);
         used = i + 1;
-        if (x & FLAG_INCL) done = true;
+        if (tag & FLAG_INCL) done = true;
       }
       if (done) break;
       j -= used;
@@ -332,62 +409,100 @@ __global__ void __launch_bounds__(SORT_THREADS)
         if (GBA_LOOKBACK_SLEEP_NS > 0) __nanosleep(GBA_LOOKBACK_SLEEP_NS);  // back off: spinning takes issue slots from the tiles it waits for
       }
     }
-    st_relaxed_u64(my, ep | FLAG_INCL | ((prefix + tile_count) & COUNT_MASK));
+#pragma unroll
+    for (int q = 0; q < DPT; ++q)
+      st_relaxed_u64(my + q, ep | FLAG_INCL | ((prefix[q] + count[q]) & COUNT_MASK));
   }
-  s_out_base[d] = g_excl + prefix;
+  s_out[tid * DPT] = g_excl + prefix[0] - t_excl;
+  if constexpr (DPT == 2)
+    s_out[tid * DPT + 1] = g_excl + hist_d[0] + prefix[DPT - 1] - (t_excl + count[0]);
   __syncthreads();
 
-  // Place keys in digit order in shared memory, then write runs of equal digits.
+  // Runs of equal digits leave in order.
 #pragma unroll
-  for (int j = 0; j < SORT_ITEMS; ++j) {
-    const int64_t idx = base + (int64_t)warp * (SORT_ITEMS * 32) + j * 32 + lane;
-    if (idx < N) {
-      const uint32_t dg = (key[j] >> shift) & (RADIX - 1);
-      const uint32_t pos = s_tile_excl[dg] + s_warp[warp][dg] + rank[j];
-      s_keys[pos] = key[j];
-      s_vals[pos] = val[j];
-    }
-  }
-  __syncthreads();
-  const int n_valid = (int)((N - base) < SORT_TILE ? (N - base) : SORT_TILE);
-  for (int i = tid; i < n_valid; i += SORT_THREADS) {
-    const uint32_t k = s_keys[i];
-    const uint32_t dg = (k >> shift) & (RADIX - 1);
-    const uint32_t out = s_out_base[dg] + ((uint32_t)i - s_tile_excl[dg]);
-    if (out < (uint32_t)N) {
-      keys_out[out] = k;
-      vals_out[out] = s_vals[i];
-    } else {
-      raise_error(err, ERR_INTERNAL);
+  for (int j = 0; j < ITEMS; ++j) {
+    const uint32_t i = (uint32_t)(tid + j * SORT_THREADS);
+    if (i < n_valid) {
+      const uint32_t k = s_keys[i];
+      const uint32_t out = s_out[(k >> shift) & mask] + i;
+      if (out < N) {
+        sp.keys_out[out] = k;
+        sp.vals_out[out] = s_vals[i];
+      } else {
+        raise_error(err, ERR_INTERNAL);
+      }
     }
   }
 }
 
+template <int ITEMS, int RADIX>
+void sweep_as(const SortPass& sp, bool first, ErrSink err, int64_t wait_ns, cudaStream_t s) {
+  constexpr int64_t TILE = ITEMS * SORT_THREADS;
+  const unsigned tiles = (unsigned)(((int64_t)sp.N + TILE - 1) / TILE);
+  if (first)
+    k_onesweep<ITEMS, RADIX, true><<<tiles, SORT_THREADS, 0, s>>>(sp, err, wait_ns);
+  else
+    k_onesweep<ITEMS, RADIX, false><<<tiles, SORT_THREADS, 0, s>>>(sp, err, wait_ns);
+}
+
 }  // namespace
 
-int sort_tiles(int64_t N) { return (int)((N + SORT_TILE - 1) / SORT_TILE); }
+SortPlan make_sort_plan(int key_bits, int max_digit_bits) {
+  SortPlan p{};
+  p.passes = (key_bits + max_digit_bits - 1) / max_digit_bits;
+  // wider digits only where they save a pass
+  const bool wide = p.passes < (key_bits + 7) / 8;
+  p.radix = wide ? 512 : 256;
+  int shift = 0;
+  for (int i = 0; i < p.passes; ++i) {  // an even split of the bits, the wider digits first
+    const int bits = (key_bits - shift + p.passes - i - 1) / (p.passes - i);
+    p.shift[i] = shift;
+    p.mask[i] = (1u << bits) - 1u;
+    shift += bits;
+  }
+  return p;
+}
+
+size_t sort_status_words(int64_t N, int radix) {
+  const int64_t small = std::min<int64_t>(N, SORT_BIG_N);
+  const int64_t tiles = std::max((small + SORT_TILE_KEYS - 1) / SORT_TILE_KEYS,
+                                 (N + 2 * SORT_TILE_KEYS - 1) / (2 * SORT_TILE_KEYS));
+  return (size_t)tiles * (size_t)radix;
+}
 
 void launch_weights(const StepArgs& a, StepScratch sc, DevStats* stats, int n_hist_words,
                     cudaStream_t s) {
   k_message_weights<<<1, 256, 0, s>>>(a, sc, stats, n_hist_words);
 }
 
-void launch_sort_histogram(const StepArgs& a, int passes, StepScratch sc, uint32_t* keys0,
-                           ErrSink err, int grid, cudaStream_t s) {
-  k_sort_histogram<<<grid, SORT_THREADS, 0, s>>>(a, passes, sc, keys0, err);
+void launch_sort_histogram(const StepArgs& a, const SortPlan& plan, uint32_t* hist,
+                           uint32_t* keys0, ErrSink err, int num_sms, cudaStream_t s) {
+  const int64_t grid = std::max<int64_t>(
+      1, std::min<int64_t>(std::max<int64_t>((a.N + 2047) / 2048,
+                                             std::min<int64_t>((a.N + 1023) / 1024, 2 * num_sms)),
+                           (int64_t)num_sms * 6));
+  if (plan.radix == 512)
+    k_sort_histogram<512><<<(unsigned)grid, SORT_THREADS, 0, s>>>(a, plan, hist, keys0, err);
+  else
+    k_sort_histogram<256><<<(unsigned)grid, SORT_THREADS, 0, s>>>(a, plan, hist, keys0, err);
 }
 
-void launch_onesweep(const StepArgs& a, bool first, int pass, const uint32_t* keys_in,
-                     const uint32_t* vals_in, uint32_t* keys_out, uint32_t* vals_out,
-                     StepScratch sc, unsigned long long* status, uint32_t epoch, ErrSink err,
-                     int64_t wait_ns, cudaStream_t s) {
-  const int tiles = sort_tiles(a.N);
-  if (first)
-    k_onesweep<true><<<tiles, SORT_THREADS, 0, s>>>(a, pass, keys_in, vals_in, keys_out,
-                                                    vals_out, sc, status, epoch, err, wait_ns);
-  else
-    k_onesweep<false><<<tiles, SORT_THREADS, 0, s>>>(a, pass, keys_in, vals_in, keys_out,
-                                                     vals_out, sc, status, epoch, err, wait_ns);
+void launch_onesweep(const SortPlan& plan, int pass, SortPass sp, ErrSink err, int64_t wait_ns,
+                     cudaStream_t s) {
+  sp.shift = plan.shift[pass];
+  sp.mask = plan.mask[pass];
+  const bool big = sp.N > SORT_BIG_N;
+  if (plan.radix == 512) {
+    if (big)
+      sweep_as<16, 512>(sp, pass == 0, err, wait_ns, s);
+    else
+      sweep_as<8, 512>(sp, pass == 0, err, wait_ns, s);
+  } else {
+    if (big)
+      sweep_as<16, 256>(sp, pass == 0, err, wait_ns, s);
+    else
+      sweep_as<8, 256>(sp, pass == 0, err, wait_ns, s);
+  }
 }
 
 }  // namespace gba

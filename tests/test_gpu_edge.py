@@ -412,12 +412,33 @@ def test_dense_sizes(D):
 
 
 def test_ragged_sort_sizes():
-    """Step sizes around the sort and segment-scan tiles (2048 positions) and
-    the classification tiles (2048 row records)."""
+    """Step sizes around the sort and segment-scan tiles (2048 positions)."""
     rng = np.random.default_rng(2)
     for n in (1, 63, 64, 65, 2047, 2048, 2049, 4095, 4096, 4097, 12289):
         cfg = cfg_of([(70_000, 8, 0, 0)], D=4, G=1)
         run_custom(cfg, [[msg(0, [rng.integers(0, 70_000, n)], [8], 4)]], max_ids=n)
+
+
+@pytest.mark.parametrize("n", [1, 2049, 300_000, 1 << 21, (1 << 21) + 4097])
+@pytest.mark.parametrize("rows", [2, 256, 257, 70_000, 1 << 18, (1 << 25) + 3, 1 << 27, (1 << 28) + 1])
+def test_sort_over_digit_widths_and_tile_sizes(n, rows):
+    """The sorted keys and their payloads (a stable order) for one to four
+    passes of 256 and of 512 counters, both tile sizes, short last tiles and
+    skewed ids."""
+    g = B.GBA([(rows, 1, 0, n, B.opt_desc(0, 0.01))], 0, None, 1, 2, iota=3, seed=1)
+    gen = torch.Generator(device="cuda").manual_seed(n + rows)
+    u = torch.rand(n, generator=gen, device="cuda", dtype=torch.float64)
+    ids = (u ** 3 * rows).to(torch.int64).clamp_(0, rows - 1)
+    ids[n // 2] = rows - 1
+    grad = torch.zeros(n, 1, device="cuda")
+    torch.cuda.synchronize()
+    g.push_ref(0, [ids], [grad], grad, 1)
+    assert g.try_apply() == 1
+    keys, occ = g.sorted_keys()
+    want = np.argsort(ids.cpu().numpy(), kind="stable")
+    assert np.array_equal(occ.astype(np.int64), want)
+    assert np.array_equal(keys.astype(np.int64), ids.cpu().numpy()[want])
+    g.close()
 
 
 # ---------------------------------------------------------------------------
