@@ -96,6 +96,7 @@ struct gba_handle {
   cudaStream_t sorts = nullptr;   // message weights, histogram, sort passes
   cudaStream_t applys = nullptr;  // segment-sum and row update
   bool overlap = false;           // consecutive steps may run concurrently
+  bool joined = true;             // the handle's stream is ordered after every step so far
   cudaEvent_t ev_pushes = nullptr;
   cudaEvent_t ev_hist[SLOTS] = {}, ev_sorted[SLOTS] = {}, ev_applied[SLOTS] = {},
               ev_densed[SLOTS] = {};
@@ -360,6 +361,8 @@ cudaError_t sync_all(gba_handle* h) {
 
 // Orders the handle's stream after every step enqueued so far.
 void join_steps(gba_handle* h) {
+  if (h->joined) return;
+  h->joined = true;
   for (int b = 0; b < SLOTS; ++b)
     if (h->slot_busy[b]) {
       cudaStreamWaitEvent(h->stream, h->ev_applied[b], 0);
@@ -1018,16 +1021,24 @@ int32_t gba_try_apply(gba_handle* h) {
     if (s != GBA_OK) return s;
   }
 
-  // ---- the step's buffers (slot b) and stream dependencies.  The sort stream
-  // runs message weights, histogram and sort passes; the handle's stream the
-  // segment-sum and row update; the side stream the dense update.
+  // ---- the step's buffers (slot b) and stream dependencies.  Message weights,
+  // histogram and sort passes go to one stream, the segment scan and row update
+  // to another, the dense update to the side stream.  Steps that may not overlap
+  // use the handle's own stream for the first two: an edge between streams costs
+  // a small step several microseconds, and there is nothing for it to allow.
   const int b = (int)(h->k & 1);
-  // everything the caller enqueued before this call (pushes included)
-  cudaEventRecord(h->ev_pushes, h->stream);
-  cudaStreamWaitEvent(h->sorts, h->ev_pushes, 0);
-  if (h->slot_busy[b]) {  // step k - 2 used these buffers
-    cudaStreamWaitEvent(h->sorts, h->ev_applied[b], 0);
-    cudaStreamWaitEvent(h->sorts, h->ev_densed[b], 0);
+  const cudaStream_t sorts = h->overlap ? h->sorts : h->stream;
+  const cudaStream_t applys = h->overlap ? h->applys : h->stream;
+  if (h->overlap) {
+    // everything the caller enqueued before this call (pushes included)
+    cudaEventRecord(h->ev_pushes, h->stream);
+    cudaStreamWaitEvent(sorts, h->ev_pushes, 0);
+    if (h->slot_busy[b]) {  // step k - 2 used these buffers
+      cudaStreamWaitEvent(sorts, h->ev_applied[b], 0);
+      cudaStreamWaitEvent(sorts, h->ev_densed[b], 0);
+    }
+  } else {
+    join_steps(h);  // steps that overlapped before the mode was turned off
   }
   StepScratch& sc = h->sc[b];
   ErrSink sink = h->sink;
@@ -1093,8 +1104,8 @@ int32_t gba_try_apply(gba_handle* h) {
                            ts.bpow2 * (double)ts.desc.opt.beta2);
     tabs[t] = tb;
   }
-  GBA_CUDA(h, cudaMemcpyAsync(dmeta, hp, h->meta_bytes, cudaMemcpyHostToDevice, h->sorts));
-  cudaEventRecord(h->meta_ev[slot], h->sorts);
+  GBA_CUDA(h, cudaMemcpyAsync(dmeta, hp, h->meta_bytes, cudaMemcpyHostToDevice, sorts));
+  cudaEventRecord(h->meta_ev[slot], sorts);
 
   StepArgs a{};
   a.k = h->k;
@@ -1119,8 +1130,8 @@ int32_t gba_try_apply(gba_handle* h) {
 
   // ---- K1: message weights (Eq. (1)); clears the per-step scratch
   {
-    Timed tm(h, GBA_K_WEIGHTS, h->sorts);
-    launch_weights(a, sc, h->d_stats, MAX_PASSES * MAX_RADIX, h->sorts);
+    Timed tm(h, GBA_K_WEIGHTS, sorts);
+    launch_weights(a, sc, h->d_stats, MAX_PASSES * MAX_RADIX, sorts);
   }
   // ---- K5 on the side stream, concurrently with the sort and segment-sum.
   // It is forked after the histogram kernel has validated every id, so a step
@@ -1131,7 +1142,7 @@ int32_t gba_try_apply(gba_handle* h) {
     const double p2 = h->dbpow2 * (double)h->dense_opt.beta2;
     DenseArgs da{h->dw, h->ds0, h->ds1, h->D, M, make_opt_step(h->dense_opt, p1, p2),
                  h->withhold_dense ? 1 : 0};
-    cudaEventRecord(h->ev_hist[b], h->sorts);
+    cudaEventRecord(h->ev_hist[b], sorts);
     cudaStreamWaitEvent(h->side, h->ev_hist[b], 0);
     if (h->eager) {  // the step's sum was accumulated at push time
       const gba_handle::EagerGroup gr = h->egroups.front();
@@ -1150,13 +1161,18 @@ int32_t gba_try_apply(gba_handle* h) {
     h->dbpow1 = p1;
     h->dbpow2 = p2;
   };
+  auto order_after_sort = [&]() {
+    if (applys == sorts) return;
+    cudaEventRecord(h->ev_sorted[b], sorts);
+    cudaStreamWaitEvent(applys, h->ev_sorted[b], 0);
+  };
   // ---- K2 sort, K3+K4 segment-sum and row update
   int final_buf = 0;
   if (N > 0) {
     {
-      Timed tm(h, GBA_K_SORT_HIST, h->sorts);
+      Timed tm(h, GBA_K_SORT_HIST, sorts);
       // the first pass writes buffer 0, so its input keys go to buffer 1
-      launch_sort_histogram(a, h->plan, sc.hist, h->d_keys[b][1], sink, h->num_sms, h->sorts);
+      launch_sort_histogram(a, h->plan, sc.hist, h->d_keys[b][1], sink, h->num_sms, sorts);
     }
     launch_dense_side();
     const uint32_t* kin = h->d_keys[b][1];
@@ -1164,7 +1180,7 @@ int32_t gba_try_apply(gba_handle* h) {
     for (int p = 0; p < h->plan.passes; ++p) {
       const int ob = p & 1;
       if (++h->epoch == 0u) h->epoch = 1u;
-      Timed tm(h, GBA_K_SORT_PASS, h->sorts);
+      Timed tm(h, GBA_K_SORT_PASS, sorts);
       SortPass sp{};
       sp.N = (uint32_t)N;
       sp.hist = sc.hist + p * h->plan.radix;
@@ -1175,13 +1191,12 @@ int32_t gba_try_apply(gba_handle* h) {
       sp.vals_out = h->d_vals[b][ob];
       sp.status = h->d_status[b];
       sp.epoch = h->epoch;
-      launch_onesweep(h->plan, p, sp, sink, h->wait_ns, h->sorts);
+      launch_onesweep(h->plan, p, sp, sink, h->wait_ns, sorts);
       kin = h->d_keys[b][ob];
       vin = h->d_vals[b][ob];
       final_buf = ob;
     }
-    cudaEventRecord(h->ev_sorted[b], h->sorts);
-    cudaStreamWaitEvent(h->applys, h->ev_sorted[b], 0);
+    order_after_sort();
     if (++h->epoch == 0u) h->epoch = 1u;
     SegOut so{};
     so.rr = h->d_rr;
@@ -1199,9 +1214,9 @@ int32_t gba_try_apply(gba_handle* h) {
     so.small_rows = h->d_small_rows;
     const SegTable* d_tabs = (const SegTable*)(dmeta + o_tabs);
     {
-      Timed tm(h, GBA_K_SEG_SCAN, h->applys);
+      Timed tm(h, GBA_K_SEG_SCAN, applys);
       launch_seg_scan(a, tabs[0], d_tabs, so, h->d_keys[b][final_buf], h->d_vals[b][final_buf],
-                      h->d_stats, sink, h->wait_ns, h->applys);
+                      h->d_stats, sink, h->wait_ns, applys);
     }
     // one pair of row kernels per range of consecutive tables of one width and
     // optimizer
@@ -1218,31 +1233,34 @@ int32_t gba_try_apply(gba_handle* h) {
       so.n_small = counters + 5;
       so.small_ticket = counters + 6;
       {
-        Timed tm(h, GBA_K_ROW_APPLY, h->applys);
-        launch_row_apply(a, r, d_tabs, so, h->d_stats, sink, h->num_sms, h->applys);
+        Timed tm(h, GBA_K_ROW_APPLY, applys);
+        launch_row_apply(a, r, d_tabs, so, h->d_stats, sink, h->num_sms, applys);
       }
       {
-        Timed tm(h, GBA_K_ROW_LONG, h->applys);
-        launch_row_long(a, r, d_tabs, so, h->d_stats, sink, h->num_sms, h->applys);
+        Timed tm(h, GBA_K_ROW_LONG, applys);
+        launch_row_long(a, r, d_tabs, so, h->d_stats, sink, h->num_sms, applys);
       }
     }
   }
   if (N == 0) {
     launch_dense_side();
-    cudaEventRecord(h->ev_sorted[b], h->sorts);
-    cudaStreamWaitEvent(h->applys, h->ev_sorted[b], 0);
+    order_after_sort();
   }
   // Adam step counts advance every global step, whether or not a row moved.
   for (auto& ts : h->tables) {
     ts.bpow1 *= (double)ts.desc.opt.beta1;
     ts.bpow2 *= (double)ts.desc.opt.beta2;
   }
-  cudaEventRecord(h->ev_applied[b], h->applys);
-  cudaEventRecord(h->ev_densed[b], h->side);
-  h->slot_busy[b] = true;
-  // Unless steps may overlap, work the caller orders after this call on its
-  // stream sees the whole step.
-  if (!h->overlap) join_steps(h);
+  if (h->overlap) {
+    cudaEventRecord(h->ev_applied[b], applys);
+    cudaEventRecord(h->ev_densed[b], h->side);
+    h->slot_busy[b] = true;
+    h->joined = false;
+  } else if (h->D > 0) {
+    // Work the caller orders after this call on its stream sees the whole step.
+    cudaEventRecord(h->ev_densed[b], h->side);
+    cudaStreamWaitEvent(h->stream, h->ev_densed[b], 0);
+  }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     h->failed = true;

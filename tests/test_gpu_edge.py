@@ -652,6 +652,31 @@ def test_pull_orders_after_overlapping_steps():
     g.close()
 
 
+def test_overlap_turned_on_and_off_between_steps():
+    """Steps enqueued in either mode, one after another without a
+    synchronisation, with pulls between them: the state of every step in order."""
+    cfg = W.reduced(2)
+    outs = []
+    for modes in ((0, 0, 0, 0, 0, 0, 0, 0), (1, 1, 0, 1, 0, 0, 1, 0)):
+        g = H.make_gpu(cfg, debug=False)
+        keep, pulled = [], []
+        for k, on in enumerate(modes):
+            g.set_overlap(bool(on))
+            msgs = W.generate_step(cfg, k, "cuda")
+            keep.append(msgs)
+            torch.cuda.current_stream().synchronize()  # the messages are there; steps run on
+            for m in msgs:
+                g.push_ref(m["token"], m["ids"], m["rows"], m["dense"], m["local_batch"])
+            assert g.try_apply() == 1
+            if k in (1, 4):
+                pulled.append(g.pull(0, msgs[0]["ids"][0]))
+        g.sync()
+        outs.append([t for t in g.table(0) + g.dense() if t is not None] + pulled)
+        g.close()
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
+
+
 def test_pull_of_an_out_of_range_id_is_latched():
     tables = [(100, 8, 0, 16, B.opt_desc())]
     g = B.GBA(tables, 0, None, 1, 4, seed=1)
