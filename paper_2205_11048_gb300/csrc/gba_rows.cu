@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, GBA_SCAN_MINB)
   __shared__ unsigned long long s_stale[2][SCAN_WARPS];
   __shared__ uint32_t s_tile;
 
+  chain_wait();
   // block-uniform: another kernel may set the word while this block reads it
   if (__syncthreads_or((ld_volatile_u32(err.step) & (ERR_ID_RANGE | ERR_TIMEOUT)) != 0u)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -632,6 +633,7 @@ __global__ void __launch_bounds__(ROW_THREADS, (CH * CPL <= 4 && !AHEAD) ? 4 : (
                 DevStats* st, ErrSink err) {
   __shared__ RowSlot s_slot[ROW_WARPS][32];
   __shared__ uint4 s_rec[ROW_WARPS][33];  // the next batch's records
+  chain_wait();
   // a failed step changes no row (warp-uniform: the warp reduces at the end)
   if (__any_sync(FULL, ld_volatile_u32(err.step) != 0u)) return;
   constexpr int P = CH * CPL;
@@ -865,6 +867,7 @@ template <int CH, int CPL, bool ADAM, bool MULTI>
 __global__ void __launch_bounds__(ROW_THREADS, 2)
     k_row_long(StepArgs a, SegTable tb0, const SegTable* tabs, int t0, int t1, SegOut so,
                DevStats* st, ErrSink err) {
+  chain_wait();
   if (__any_sync(FULL, ld_volatile_u32(err.step) != 0u)) return;
   constexpr int P = CH * CPL;
   constexpr int UNR = P <= 4 ? 8 : 4;
@@ -1046,8 +1049,8 @@ void launch_apply_as(const StepArgs& a, const RowRange& r, const SegTable* tabs,
   // every warp has at least the rows that it works on at once
   const int64_t want = (r.n + ROW_WARPS * G - 1) / (ROW_WARPS * G);
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms * bps, want));
-  k_row_apply<CH, CPL, ADAM, MULTI, AHEAD>
-      <<<(unsigned)grid, ROW_THREADS, 0, s>>>(a, r.first, tabs, r.t0, r.t1, so, stats, err);
+  launch_chained(a.N, k_row_apply<CH, CPL, ADAM, MULTI, AHEAD>, (unsigned)grid, ROW_THREADS, 0, s, a,
+                 r.first, tabs, r.t0, r.t1, so, stats, err);
 }
 
 template <int CH, int CPL, bool ADAM, bool MULTI>
@@ -1068,8 +1071,8 @@ void launch_rows_as(const StepArgs& a, const RowRange& r, const SegTable* tabs, 
     const int64_t warps = r.n / ((LONG_ROW + 1) * G) + r.n / SMALL_MAX + 1;
     const int64_t grid = std::max<int64_t>(
         1, std::min<int64_t>((int64_t)num_sms * bps, (warps + ROW_WARPS - 1) / ROW_WARPS));
-    k_row_long<CH, CPL, ADAM, MULTI>
-        <<<(unsigned)grid, ROW_THREADS, 0, s>>>(a, r.first, tabs, r.t0, r.t1, so, stats, err);
+    launch_chained(a.N, k_row_long<CH, CPL, ADAM, MULTI>, (unsigned)grid, ROW_THREADS, 0, s, a, r.first,
+                   tabs, r.t0, r.t1, so, stats, err);
   }
 }
 
@@ -1091,8 +1094,8 @@ template <bool MULTI, bool CACHED, bool UNIT>
 void launch_scan_as(const StepArgs& a, const SegTable& tb0, const SegTable* tabs, const SegOut& so,
                     const uint32_t* keys, const uint32_t* vals, DevStats* stats, ErrSink err,
                     int64_t wait_ns, size_t smem, cudaStream_t s) {
-  k_seg_scan<MULTI, CACHED, UNIT><<<(unsigned)scan_tiles(a.N), SCAN_THREADS, smem, s>>>(
-      a, tb0, tabs, so, keys, vals, stats, err, wait_ns);
+  launch_chained(a.N, k_seg_scan<MULTI, CACHED, UNIT>, (unsigned)scan_tiles(a.N), SCAN_THREADS, smem, s,
+                 a, tb0, tabs, so, keys, vals, stats, err, wait_ns);
 }
 
 }  // namespace

@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
   __shared__ uint32_t s_nb[TAB_CACHE + 1];
   const int tid = threadIdx.x;
   for (int i = tid; i < MAX_PASSES * RADIX; i += SORT_THREADS) (&h[0][0])[i] = 0u;
+  chain_wait();
   const int T = a.T, M = a.M;
   const bool offs_cached = T * (M + 1) <= OFF_CACHE, tabs_cached = T <= TAB_CACHE;
   if (offs_cached)
@@ -232,14 +233,15 @@ __global__ void __launch_bounds__(SORT_THREADS, ITEMS == 8 ? 5 : 4)
   __shared__ uint32_t s_vals[TILE];
   __shared__ uint32_t s_tile;
 
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t* cnt_words = reinterpret_cast<uint32_t*>(&s_cnt[0][0]);
+  for (int i = tid; i < SORT_WARPS * RADIX / 2; i += SORT_THREADS) cnt_words[i] = 0u;
+  chain_wait();
   // An id range error was latched before this launch (by the histogram):
   // every tile of every pass skips, consistently.
   if (__syncthreads_or((ld_volatile_u32(err.step) & ERR_ID_RANGE) != 0u)) return;
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) s_tile = atomicAdd(sp.ticket, 1u);
-  uint32_t* cnt_words = reinterpret_cast<uint32_t*>(&s_cnt[0][0]);
-  for (int i = tid; i < SORT_WARPS * RADIX / 2; i += SORT_THREADS) cnt_words[i] = 0u;
   uint32_t hist_d[DPT];
 #pragma unroll
   for (int q = 0; q < DPT; ++q) hist_d[q] = sp.hist[tid * DPT + q];
@@ -440,9 +442,9 @@ void sweep_as(const SortPass& sp, bool first, ErrSink err, int64_t wait_ns, cuda
   constexpr int64_t TILE = ITEMS * SORT_THREADS;
   const unsigned tiles = (unsigned)(((int64_t)sp.N + TILE - 1) / TILE);
   if (first)
-    k_onesweep<ITEMS, RADIX, true><<<tiles, SORT_THREADS, 0, s>>>(sp, err, wait_ns);
+    launch_chained(sp.N, k_onesweep<ITEMS, RADIX, true>, tiles, SORT_THREADS, 0, s, sp, err, wait_ns);
   else
-    k_onesweep<ITEMS, RADIX, false><<<tiles, SORT_THREADS, 0, s>>>(sp, err, wait_ns);
+    launch_chained(sp.N, k_onesweep<ITEMS, RADIX, false>, tiles, SORT_THREADS, 0, s, sp, err, wait_ns);
 }
 
 }  // namespace
@@ -482,9 +484,9 @@ void launch_sort_histogram(const StepArgs& a, const SortPlan& plan, uint32_t* hi
                                              std::min<int64_t>((a.N + 1023) / 1024, 2 * num_sms)),
                            (int64_t)num_sms * 6));
   if (plan.radix == 512)
-    k_sort_histogram<512><<<(unsigned)grid, SORT_THREADS, 0, s>>>(a, plan, hist, keys0, err);
+    launch_chained(a.N, k_sort_histogram<512>, (unsigned)grid, SORT_THREADS, 0, s, a, plan, hist, keys0, err);
   else
-    k_sort_histogram<256><<<(unsigned)grid, SORT_THREADS, 0, s>>>(a, plan, hist, keys0, err);
+    launch_chained(a.N, k_sort_histogram<256>, (unsigned)grid, SORT_THREADS, 0, s, a, plan, hist, keys0, err);
 }
 
 void launch_onesweep(const SortPlan& plan, int pass, SortPass sp, ErrSink err, int64_t wait_ns,
