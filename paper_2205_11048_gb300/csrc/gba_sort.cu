@@ -209,8 +209,11 @@ __global__ void __launch_bounds__(SORT_THREADS)
 // about four warp instructions of 32.  Keys and payloads go to shared memory in
 // digit order before the look-back, so that few registers live through it (48
 // instead of 80: five blocks per SM instead of three); a short last tile is
-// padded with the largest key, which needs no checks; match.any groups equal
-// digits (ballots per bit: 1.12 ms a pass against 0.83 on 131M keys).  Above
+// padded with the largest key, which needs no checks.  Lanes of equal digits find
+// each other through a shared word of lane bits per digit in the first pass, where
+// digits come in no order (975 us against 1,097 with match.any on 131M keys), and
+// by match.any in the later ones, where hot keys come in runs that would meet in
+// one word (1,083 us against 824; ballots per bit 1,123).  Above
 // SORT_BIG_N keys a tile holds 4,096 of them (5.2M keys: 70 us a pass against 89
 // with 2,048).  Digits are 8 bits wide, or up to 9 where that saves a pass: 26-bit
 // keys take three passes.  131M keys: 4 x 1.46 -> 1.12 + 2 x 0.83 ms.
@@ -226,16 +229,19 @@ __global__ void __launch_bounds__(SORT_THREADS, ITEMS == 8 ? 5 : 4)
   constexpr int WIN = DPT == 1 ? 8 : 4;      // look-back window
   static_assert(DPT == 1 || DPT == 2, "one or two digits per thread");
   __shared__ __align__(4) uint16_t s_cnt[SORT_WARPS][RADIX];  // per-warp digit counts, then offsets
-  __shared__ uint32_t s_excl[RADIX];  // first tile slot of each digit
   __shared__ uint32_t s_out[RADIX];   // output position of tile slot 0 of each digit
   __shared__ uint32_t s_tmp[2][SORT_WARPS];
-  __shared__ uint32_t s_keys[TILE];
-  __shared__ uint32_t s_vals[TILE];
+  __shared__ uint32_t s_kv[2 * TILE];
+  uint32_t* const s_keys = s_kv;
+  uint32_t* const s_vals = s_kv + TILE;
+  static_assert(SORT_WARPS * RADIX <= 2 * TILE, "a word of lane bits per warp and digit");
   __shared__ uint32_t s_tile;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t* cnt_words = reinterpret_cast<uint32_t*>(&s_cnt[0][0]);
   for (int i = tid; i < SORT_WARPS * RADIX / 2; i += SORT_THREADS) cnt_words[i] = 0u;
+  if (FIRST)
+    for (int i = tid; i < SORT_WARPS * RADIX; i += SORT_THREADS) s_kv[i] = 0u;
   chain_wait();
   // An id range error was latched before this launch (by the histogram):
   // every tile of every pass skips, consistently.
@@ -275,15 +281,26 @@ __global__ void __launch_bounds__(SORT_THREADS, ITEMS == 8 ? 5 : 4)
   // Warp-level multi-split: stable rank of each key among equal digits.
   const uint32_t lt = lanemask_lt();
   uint32_t rank[ITEMS / 2];  // two 16-bit ranks each
+  uint32_t* lanes = s_kv + warp * RADIX;  // the places of the keys are still free
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) {
     const uint32_t d = (key[j] >> shift) & mask;
-    const uint32_t peers = __match_any_sync(FULL, d);
+    uint32_t peers;
+    if (FIRST) {
+      atomicOr(lanes + d, 1u << lane);
+      __syncwarp();
+      peers = lanes[d];
+    } else {
+      peers = __match_any_sync(FULL, d);
+    }
     const uint32_t before = s_cnt[warp][d];
     const uint32_t r = before + __popc(peers & lt);
     rank[j / 2] = (j & 1) ? rank[j / 2] | (r << 16) : r;
     __syncwarp();
-    if ((peers & lt) == 0u) s_cnt[warp][d] = (uint16_t)(before + __popc(peers));
+    if ((peers & lt) == 0u) {
+      s_cnt[warp][d] = (uint16_t)(before + __popc(peers));
+      if (FIRST) lanes[d] = 0u;
+    }
     __syncwarp();
   }
   __syncthreads();
@@ -349,8 +366,15 @@ __global__ void __launch_bounds__(SORT_THREADS, ITEMS == 8 ? 5 : 4)
       t_excl += s_tmp[0][w];
       g_excl += s_tmp[1][w];
     }
-  s_excl[tid * DPT] = t_excl;
-  if constexpr (DPT == 2) s_excl[tid * DPT + 1] = t_excl + count[0];
+  // the warps' offsets within the tile
+  if constexpr (DPT == 1) {
+#pragma unroll
+    for (int w = 0; w < SORT_WARPS; ++w) s_cnt[w][tid] = (uint16_t)(s_cnt[w][tid] + t_excl);
+  } else {
+    const uint32_t both = t_excl | (t_excl + count[0]) << 16;
+#pragma unroll
+    for (int w = 0; w < SORT_WARPS; ++w) cnt_words[w * (RADIX / 2) + tid] += both;
+  }
   __syncthreads();
 
   // Keys and payloads in digit order in shared memory.
@@ -358,7 +382,7 @@ __global__ void __launch_bounds__(SORT_THREADS, ITEMS == 8 ? 5 : 4)
   for (int j = 0; j < ITEMS; ++j) {
     const uint32_t d = (key[j] >> shift) & mask;
     const uint32_t r = (j & 1) ? rank[j / 2] >> 16 : rank[j / 2] & 0xFFFFu;
-    const uint32_t pos = s_excl[d] + s_cnt[warp][d] + r;
+    const uint32_t pos = s_cnt[warp][d] + r;
     s_keys[pos] = key[j];
     s_vals[pos] = val[j];
   }
