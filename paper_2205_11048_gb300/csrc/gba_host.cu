@@ -533,10 +533,10 @@ gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
     h->d_items = nullptr;
     const int64_t stiles = scan_tiles(cap);
     const int64_t long_cap = cap / (LONG_ROW + 1) + h->T + 1;
-    const int64_t items_cap = cap / MIN_CHUNK + long_cap;
+    const int64_t items_cap = long_items(cap, h->num_sms) + long_cap;
     int64_t part_floats = 1;  // of the widest range of tables
     for (const TableState& ts : h->tables)
-      part_floats = std::max(part_floats, long_parts(cap, ts.desc.dim) * ts.desc.dim);
+      part_floats = std::max(part_floats, long_parts(cap, ts.desc.dim, h->num_sms) * ts.desc.dim);
     GBA_CUDA(h, cudaMalloc(&h->d_rr, (size_t)(cap + h->T + 1) * sizeof(uint4)));
     GBA_CUDA(h, cudaMalloc(&h->d_kl, (size_t)cap * sizeof(float*)));
     GBA_CUDA(h, cudaMalloc(&h->d_kw, (size_t)cap * sizeof(float)));

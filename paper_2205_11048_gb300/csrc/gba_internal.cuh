@@ -513,15 +513,16 @@ constexpr int LONG_ROW = 4;
 #endif
 constexpr int SMALL_MAX = GBA_SMALL_MAX;
 static_assert(SMALL_MAX < 256, "a small row's count shares a word with its table");
-constexpr int MIN_CHUNK = 128;  // least kept occurrences per chunk of a long row
 #ifndef GBA_SCAN_TILE
 #define GBA_SCAN_TILE 2048
 #endif
 constexpr int SCAN_TILE = GBA_SCAN_TILE;  // sorted positions per segment-scan tile
 
 int64_t scan_tiles(int64_t N);
-// The most chunk-sum slots that n occurrences of rows of width d can need.
-int64_t long_parts(int64_t n, int d);
+// The most chunks, beside one for each long row, that n occurrences can make, and
+// the most chunk-sum slots that they can need at width d.
+int64_t long_items(int64_t n, int num_sms);
+int64_t long_parts(int64_t n, int d, int num_sms);
 
 // tb0: the first table; tabs: all of them, on the device.
 void launch_seg_scan(const StepArgs& a, const SegTable& tb0, const SegTable* tabs,

@@ -562,6 +562,8 @@ __device__ __forceinline__ void add_part(CSum (&acc)[CH * CPL], bool unit, float
   for (int i = 0; i < CH * CPL; ++i) csum_add_w(acc[i], unit, f, g.v[i]);
 }
 
+constexpr int LONG_WARPS = 16;  // of k_row_long per SM
+
 // Lanes per row (a power of two) and rows per warp of a width of C pieces.
 __host__ __device__ inline int row_lanes(int C, int CPL) {
   int L = 1;
@@ -569,10 +571,18 @@ __host__ __device__ inline int row_lanes(int C, int CPL) {
   return L;
 }
 
-// Kept occurrences per chunk of a row longer than SMALL_MAX: 64 for each of
-// the warp's lane groups, at least 128.
-__host__ __device__ inline uint32_t chunk_entries(int L) {
-  return L >= 16 ? 128u : 64u * (uint32_t)(32 / L);
+// Kept occurrences per chunk of a row longer than SMALL_MAX, for a range of
+// tables with n occurrences whose rows take L lanes: 64 for each of the
+// warp's lane groups (128 for a group of 32), and fewer, down to 32, while there
+// would not be two chunks for every warp that can run: such a step's time is that of
+// its longest chunk (steps of 0.33M ids x 256 floats 328 -> 314 us, of 0.85M x 32 199
+// -> 195).  Chunks of 8 or 16 a group cost more in claims and partial sums than they
+// save (0.17M ids x 18 floats: 398 -> 410 us with 8; 0.03M x 16: 52.4 -> 53.7 with 16).
+inline uint32_t chunk_entries(int64_t n, int L, int num_sms) {
+  const int64_t G = 32 / L;
+  int64_t per = L == 32 ? 128 : 64;  // entries per lane group
+  while (per > 32 && n < per * G * 2 * num_sms * LONG_WARPS) per >>= 1;
+  return (uint32_t)(per * G);
 }
 
 // The table of row record u among tables [t0, t1).
@@ -629,8 +639,8 @@ struct RowRegs {
 
 template <int CH, int CPL, bool ADAM, bool MULTI, bool AHEAD>
 __global__ void __launch_bounds__(ROW_THREADS, (CH * CPL <= 4 && !AHEAD) ? 4 : (CPL <= 2 ? 3 : 2))
-    k_row_apply(StepArgs a, SegTable tb0, const SegTable* tabs, int t0, int t1, SegOut so,
-                DevStats* st, ErrSink err) {
+    k_row_apply(StepArgs a, SegTable tb0, const SegTable* tabs, int t0, int t1, uint32_t chunk,
+                SegOut so, DevStats* st, ErrSink err) {
   __shared__ RowSlot s_slot[ROW_WARPS][32];
   __shared__ uint4 s_rec[ROW_WARPS][33];  // the next batch's records
   chain_wait();
@@ -649,7 +659,6 @@ __global__ void __launch_bounds__(ROW_THREADS, (CH * CPL <= 4 && !AHEAD) ? 4 : (
   const bool unit = a.decay == 0;  // every kept weight is 1
   const int mode = a.sparse_den;
   const int32_t tag = (int32_t)(a.k + 1);
-  const uint32_t chunk = chunk_entries(L);
   RowSlot* slot = s_slot[warp];
   uint32_t applied = 0u;
 
@@ -865,8 +874,8 @@ __device__ __forceinline__ void sum_entries(const SegOut& so, bool unit, uint32_
 
 template <int CH, int CPL, bool ADAM, bool MULTI>
 __global__ void __launch_bounds__(ROW_THREADS, 2)
-    k_row_long(StepArgs a, SegTable tb0, const SegTable* tabs, int t0, int t1, SegOut so,
-               DevStats* st, ErrSink err) {
+    k_row_long(StepArgs a, SegTable tb0, const SegTable* tabs, int t0, int t1, uint32_t chunk,
+               SegOut so, DevStats* st, ErrSink err) {
   chain_wait();
   if (__any_sync(FULL, ld_volatile_u32(err.step) != 0u)) return;
   constexpr int P = CH * CPL;
@@ -880,7 +889,6 @@ __global__ void __launch_bounds__(ROW_THREADS, 2)
   const int g = lane >> lg, l = lane & (L - 1);
   const bool unit = a.decay == 0;  // every kept weight is 1
   const int32_t tag = (int32_t)(a.k + 1);
-  const uint32_t chunk = chunk_entries(L);
   uint32_t applied = 0u;
   auto claim = [&](uint32_t* ticket, uint32_t n) {
     uint32_t v = 0u;
@@ -1050,7 +1058,8 @@ void launch_apply_as(const StepArgs& a, const RowRange& r, const SegTable* tabs,
   const int64_t want = (r.n + ROW_WARPS * G - 1) / (ROW_WARPS * G);
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms * bps, want));
   launch_chained(a.N, k_row_apply<CH, CPL, ADAM, MULTI, AHEAD>, (unsigned)grid, ROW_THREADS, 0, s, a,
-                 r.first, tabs, r.t0, r.t1, so, stats, err);
+                 r.first, tabs, r.t0, r.t1, chunk_entries(r.n, (int)(32 / G), num_sms), so, stats,
+                 err);
 }
 
 template <int CH, int CPL, bool ADAM, bool MULTI>
@@ -1072,7 +1081,7 @@ void launch_rows_as(const StepArgs& a, const RowRange& r, const SegTable* tabs, 
     const int64_t grid = std::max<int64_t>(
         1, std::min<int64_t>((int64_t)num_sms * bps, (warps + ROW_WARPS - 1) / ROW_WARPS));
     launch_chained(a.N, k_row_long<CH, CPL, ADAM, MULTI>, (unsigned)grid, ROW_THREADS, 0, s, a, r.first,
-                   tabs, r.t0, r.t1, so, stats, err);
+                   tabs, r.t0, r.t1, chunk_entries(r.n, (int)(32 / G), num_sms), so, stats, err);
   }
 }
 
@@ -1102,9 +1111,17 @@ void launch_scan_as(const StepArgs& a, const SegTable& tb0, const SegTable* tabs
 
 int64_t scan_tiles(int64_t N) { return (N + SCAN_TILE - 1) / SCAN_TILE; }
 
-int64_t long_parts(int64_t n, int d) {
+int64_t long_items(int64_t n, int num_sms) {
+  // beside one per row: full chunks, or those of a step with few
+  return n / 128 + 4 * (int64_t)num_sms * LONG_WARPS + 1;
+}
+
+int64_t long_parts(int64_t n, int d, int num_sms) {
   const int CPL = (d & 3) == 0 ? (d <= 128 ? 1 : 2) : (d <= 32 ? 1 : d <= 64 ? 2 : d <= 128 ? 4 : 8);
-  return 2 * (n / chunk_entries(row_lanes((d & 3) == 0 ? d / 4 : d, CPL))) + 1;
+  const int L = row_lanes((d & 3) == 0 ? d / 4 : d, CPL);
+  // chunks of full size, or smaller ones in a step of at most twice the chunks
+  // that the warps take at a time (twice that after the last halving)
+  return 2 * (n / (32 / L * (L == 32 ? 128 : 64))) + 2 * 4 * (int64_t)num_sms * LONG_WARPS + 1;
 }
 
 void launch_seg_scan(const StepArgs& a, const SegTable& tb0, const SegTable* tabs,

@@ -326,12 +326,28 @@ def test_kept_count_boundaries_of_the_row_kernels(dim, rule):
     run_custom(cfg, steps, rule=rule)
 
 
-@pytest.mark.parametrize("dim,chunk", [(4, 2048), (8, 1024), (13, 128), (16, 512), (28, 256), (132, 128)])
-def test_chunk_boundaries_of_long_rows(dim, chunk):
+def chunk_of(n, dim):
+    """Kept occurrences per chunk of a long row in a step of n occurrences."""
+    pieces = dim // 4 if dim % 4 == 0 else dim
+    lanes = min(32, 1 << (pieces - 1).bit_length())
+    groups, warps = 32 // lanes, 16 * torch.cuda.get_device_properties(0).multi_processor_count
+    per = 128 if lanes == 32 else 64
+    while per > 32 and n < per * groups * 2 * warps:
+        per //= 2
+    return per * groups
+
+
+@pytest.mark.parametrize("dim,n", [(4, 0), (8, 0), (13, 0), (16, 0), (28, 0), (132, 0), (16, 350_000),
+                                   (36, 200_000), (64, 640_000), (100, 320_000), (129, 640_000)])
+def test_chunk_boundaries_of_long_rows(dim, n):
     """Rows with kept occurrences on each side of one and of several chunks,
-    whose size depends on the width, and one with more chunks than a lane group
-    merges at a time."""
-    counts = [chunk - 1, chunk, chunk + 1, 2 * chunk, 2 * chunk + 1, 37 * chunk + 3, 1, 33]
+    whose size depends on the width and on the step's occurrences (short rows
+    make up the number), and one with more chunks than the lane groups merge at
+    a time."""
+    c = chunk_of(n, dim)
+    counts = [c - 1, c, c + 1, 2 * c, 2 * c + 1, 37 * c + 3, 1, 33, 34]
+    counts += [4] * max(0, (n - sum(counts)) // 4)
+    assert chunk_of(sum(counts), dim) in (c, 2 * c)
     M, D = 3, 5
     rng = np.random.default_rng(dim)
     cfg = cfg_of([(len(counts) + 2, dim, 0, 0)], D=D, G=M, iota=1)
@@ -342,7 +358,7 @@ def test_chunk_boundaries_of_long_rows(dim, chunk):
         return [msg(max(0, k - 2 * (m == 1)), [part], [dim], D, scale=0.001)
                 for m, part in enumerate(np.split(ids, cut))]
 
-    run_custom(cfg, [batch(0), batch(1), batch(2)], max_ids=60 * chunk + 200)
+    run_custom(cfg, [batch(0), batch(1), batch(2)], max_ids=sum(counts))
 
 
 def test_tables_that_share_launches():
