@@ -31,6 +31,7 @@
 // and chunks), so results are bit-identical run to run; no float atomics
 // anywhere.  Sums are compensated (TwoSum).
 #include <algorithm>
+#include <type_traits>
 
 #include "gba_internal.cuh"
 
@@ -104,10 +105,11 @@ __device__ __forceinline__ float row_denominator(int mode, uint32_t c_all, uint3
 // Bound by instruction issue and by the wait for earlier tiles: 8 B are read
 // and at most 28 written per position, about seven warp instructions.  Message
 // offsets, addresses and 32-bit tokens sit in shared memory, a message is found
-// by an even-split guess and a step or two, and a round of the look-back only
-// settles how far it reaches: the counts are added up per thread and reduced
+// by an even-split guess and a step or two, a tile within one table uses that
+// table's fields throughout, and a round of the look-back only settles how far it
+// reaches: the counts are added up per thread and reduced
 // once.  0.85M positions 40 -> 18 us, 5.2M (200 MB of tags) 197 -> 100, 131M in
-// four tables 3.12 -> 1.80 ms.
+// four tables 3.12 -> 1.4 ms.
 // ---------------------------------------------------------------------------
 #ifndef GBA_LOOKBACK_SLEEP_NS
 #define GBA_LOOKBACK_SLEEP_NS 64
@@ -176,103 +178,115 @@ __global__ void __launch_bounds__(SCAN_THREADS, GBA_SCAN_MINB)
     key_prev = keys[pw - 1];
     val_prev = vals[pw - 1];
   }
-  // the table of this lane's first position; later ones only move up
-  int t_first = 0;
-  if (MULTI && key[0] != NO_KEY) {
+  // The table of the tile's first position, whose fields the whole tile then
+  // uses; a tile that runs into the next table (mixed) looks its positions'
+  // tables up one by one, each lane moving up from that of its first.
+  int t_one = 0;
+  if (MULTI) {
     int lo = 0, hi = T;
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
-      if (tabs[mid].key_base <= key[0])
+      if (tabs[mid].nb <= tile * (uint32_t)SCAN_TILE)
         lo = mid;
       else
         hi = mid;
     }
-    t_first = lo;
+    t_one = lo;
   }
+  const SegTable& tb1 = MULTI ? tabs[t_one] : tb0;
+  const bool mixed = MULTI && min((tile + 1u) * (uint32_t)SCAN_TILE, N) > tb1.nb + tb1.n;
   auto advance = [&](int t, uint32_t k) {
     while (t + 1 < T && tabs[t + 1].key_base <= k) ++t;
     return t;
   };
-  auto tab = [&](int t) -> const SegTable& { return MULTI ? tabs[t] : tb0; };
-  // the rows' step tags, all loads in flight together (positions of one row
-  // read the same tag, so only a row's first read reaches DRAM)
   int32_t tg[SCAN_ITEMS];
-  {
-    int t = t_first;
-#pragma unroll
-    for (int j = 0; j < SCAN_ITEMS; ++j) {
-      tg[j] = (int32_t)a.k;  // message staleness: against the current step
-      if (key[j] != NO_KEY) {
-        if (MULTI) t = advance(t, key[j]);
-        const uint32_t x = key[j] - tab(t).key_base;
-        if (a.row_staleness == 0 && x < tab(t).rows) tg[j] = __ldg(tab(t).ver + x);
-      }
-    }
-  }
-
-  // ---- pass 1: decide every position
   float f_[UNIT ? 1 : SCAN_ITEMS];
   uint32_t flags = 0u;  // bit 4j: head, 4j+1: keep, 4j+2: new (message, row) pair
   uint32_t cnt[4] = {0u, 0u, 0u, 0u};  // the warp's totals
   unsigned long long stale_sum = 0ull;
   uint32_t stale_max = 0u;
-  int m_last = -1;  // message of the position before this round's first
-  if (key_prev != NO_KEY) {
-    // only compared with positions of the same row, so lane 0's table serves
-    const int t0 = MULTI ? __shfl_sync(FULL, t_first, 0) : 0;
-    uint32_t o = val_prev - tab(t0).nb;
-    if (o < tab(t0).n) m_last = message_of(off_all + (size_t)t0 * (M + 1), M, o, tab(t0).mscale);
-  }
-  {
-    int t = t_first;
-#pragma unroll
-    for (int j = 0; j < SCAN_ITEMS; ++j) {
-      bool in = key[j] != NO_KEY;
-      if (MULTI && in) t = advance(t, key[j]);
-      const SegTable& tb = tab(t);
-      const uint32_t x = key[j] - tb.key_base;
-      uint32_t o = val[j] - tb.nb;
-      if (in && (o >= tb.n || x >= tb.rows)) {
-        raise_error(err, ERR_INTERNAL);  // cannot happen for a correctly sorted array
-        in = false;
-      }
-      int m = -1;
-      if (in) m = message_of(off_all + (size_t)t * (M + 1), M, o, tb.mscale);
-      uint32_t kp = __shfl_up_sync(FULL, key[j], 1);
-      int mp = __shfl_up_sync(FULL, m, 1);
-      if (lane == 0) {
-        kp = key_prev;
-        mp = m_last;
-      }
-      key_prev = __shfl_sync(FULL, key[j], 31);
-      m_last = __shfl_sync(FULL, m, 31);
-      bool head = false, keep = false, newp = false;
-      float f = 0.f;
-      if (in) {
-        head = key[j] != kp;
-        newp = head || m != mp;
-        const int32_t tk = CACHED ? tok32[m] : token32(a.tokens[m]);
-        const uint32_t sl = tg[j] > tk ? (uint32_t)(tg[j] - tk) : 0u;
-        if (UNIT) {
-          keep = sl <= (uint32_t)a.iota && m < hop_limit;
-        } else {
-          f = m < hop_limit ? decay_weight(a, sl) : 0.f;
-          keep = f > 0.f;
-        }
-        if (newp) {
-          stale_sum += sl;
-          stale_max = max(stale_max, sl);
+  auto decide = [&](auto mixed_tag) {
+  constexpr bool MIX = decltype(mixed_tag)::value;
+    // the rows' step tags, all loads in flight together (positions of one row
+    // read the same tag, so only a row's first read reaches DRAM)
+    {
+      int t = t_one;
+  #pragma unroll
+      for (int j = 0; j < SCAN_ITEMS; ++j) {
+        tg[j] = (int32_t)a.k;  // message staleness: against the current step
+        if (key[j] != NO_KEY) {
+          if (MIX) t = advance(t, key[j]);
+          const uint32_t x = key[j] - (MIX ? tabs[t] : tb1).key_base;
+          if (a.row_staleness == 0 && x < (MIX ? tabs[t] : tb1).rows) tg[j] = __ldg((MIX ? tabs[t] : tb1).ver + x);
         }
       }
-      tg[j] = m;  // the tag has served; the message is needed in pass 2,
-      val[j] = o;  // and the occurrence's place in it
-      if (!UNIT) f_[UNIT ? 0 : j] = f;
-      flags |= ((head ? 1u : 0u) | (keep ? 2u : 0u) | (newp ? 4u : 0u)) << (4 * j);
-      cnt[0] += __popc(__ballot_sync(FULL, head));
-      cnt[1] += __popc(__ballot_sync(FULL, keep));
-      cnt[2] += __popc(__ballot_sync(FULL, newp));
-      cnt[3] += __popc(__ballot_sync(FULL, newp && keep));
     }
+  
+    // ---- pass 1: decide every position
+    int m_last = -1;  // message of the position before this round's first
+    if (key_prev != NO_KEY) {
+      // only compared with positions of the same row, so lane 0's table serves
+      const int t0 = MIX ? __shfl_sync(FULL, advance(t_one, key[0]), 0) : t_one;
+      const SegTable& tb = MIX ? tabs[t0] : tb1;
+      uint32_t o = val_prev - tb.nb;
+      if (o < tb.n) m_last = message_of(off_all + (size_t)t0 * (M + 1), M, o, tb.mscale);
+    }
+    {
+      int t = t_one;
+  #pragma unroll
+      for (int j = 0; j < SCAN_ITEMS; ++j) {
+        bool in = key[j] != NO_KEY;
+        if (MIX && in) t = advance(t, key[j]);
+        const SegTable& tb = (MIX ? tabs[t] : tb1);
+        const uint32_t x = key[j] - tb.key_base;
+        uint32_t o = val[j] - tb.nb;
+        if (in && (o >= tb.n || x >= tb.rows)) {
+          raise_error(err, ERR_INTERNAL);  // cannot happen for a correctly sorted array
+          in = false;
+        }
+        int m = -1;
+        if (in) m = message_of(off_all + (size_t)t * (M + 1), M, o, tb.mscale);
+        // the position before: the lane below, for lane 0 the last of the round before
+        const uint32_t kp = __shfl_sync(FULL, lane == 31 ? key_prev : key[j], (lane + 31) & 31);
+        const int mp = __shfl_sync(FULL, lane == 31 ? m_last : m, (lane + 31) & 31);
+        key_prev = key[j];
+        m_last = m;
+        bool head = false, keep = false, newp = false;
+        float f = 0.f;
+        if (in) {
+          head = key[j] != kp;
+          newp = head || m != mp;
+          const int32_t tk = CACHED ? tok32[m] : token32(a.tokens[m]);
+          const uint32_t sl = tg[j] > tk ? (uint32_t)(tg[j] - tk) : 0u;
+          if (UNIT) {
+            keep = sl <= (uint32_t)a.iota && m < hop_limit;
+          } else {
+            f = m < hop_limit ? decay_weight(a, sl) : 0.f;
+            keep = f > 0.f;
+          }
+          if (newp) {
+            stale_sum += sl;
+            stale_max = max(stale_max, sl);
+          }
+        }
+        tg[j] = m;  // the tag has served; the message is needed in pass 2,
+        val[j] = o;  // and the occurrence's place in it
+        if (!UNIT) f_[UNIT ? 0 : j] = f;
+        flags |= ((head ? 1u : 0u) | (keep ? 2u : 0u) | (newp ? 4u : 0u)) << (4 * j);
+        cnt[0] += __popc(__ballot_sync(FULL, head));
+        cnt[1] += __popc(__ballot_sync(FULL, keep));
+        cnt[2] += __popc(__ballot_sync(FULL, newp));
+        cnt[3] += __popc(__ballot_sync(FULL, newp && keep));
+      }
+    }
+  };
+  if constexpr (MULTI) {
+    if (mixed)
+      decide(std::true_type{});
+    else
+      decide(std::false_type{});
+  } else {
+    decide(std::false_type{});
   }
 
   // ---- the warps' exclusive prefixes within the tile, the tile's totals
@@ -379,7 +393,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, GBA_SCAN_MINB)
         const uint32_t U = pre[0] + tile_tot[0];
         so.rr[U] = make_uint4(0u, pre[1] + tile_tot[1], pre[2] + tile_tot[2], pre[3] + tile_tot[3]);
         so.ustart[T] = U;
-        for (int t = T - 1; t >= 0 && tab(t).n == 0u; --t) so.ustart[t] = U;
+        for (int t = T - 1; MULTI && t >= 0 && tabs[t].n == 0u; --t) so.ustart[t] = U;
         // the step's counters of Table 3's kind
         atomicAdd(&st->rows_touched, (unsigned long long)U);
         atomicAdd(&st->occ_kept, (unsigned long long)(pre[1] + tile_tot[1]));
@@ -401,16 +415,18 @@ __global__ void __launch_bounds__(SCAN_THREADS, GBA_SCAN_MINB)
   // ---- pass 2: row records and the kept list, in order
 #pragma unroll
   for (int c = 0; c < 4; ++c) run[c] += s_base[c];
+  auto emit = [&](auto mixed_tag) {
+    constexpr bool MIX = decltype(mixed_tag)::value;
   {
-    int t = t_first;
+    int t = t_one;
 #pragma unroll
     for (int j = 0; j < SCAN_ITEMS; ++j) {
       const uint32_t fl = (flags >> (4 * j)) & 7u;
       const bool head = fl & 1u, keep = fl & 2u, newp = fl & 4u;
       const uint32_t hm = __ballot_sync(FULL, head), km = __ballot_sync(FULL, keep),
                      nm = __ballot_sync(FULL, newp);
-      if (MULTI && key[j] != NO_KEY) t = advance(t, key[j]);
-      const SegTable& tb = tab(t);
+      if (MIX && key[j] != NO_KEY) t = advance(t, key[j]);
+      const SegTable& tb = MIX ? tabs[t] : tb1;
       const uint32_t k_at = run[1] + __popc(km & lt);
       if (head) {
         const uint32_t u = run[0] + __popc(hm & lt);
@@ -419,7 +435,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, GBA_SCAN_MINB)
         // the first row of a table (and of the empty tables before it)
         if (pw + j * 32 + lane == tb.nb) {
           so.ustart[t] = u;
-          for (int e = t - 1; MULTI && e >= 0 && tab(e).n == 0u; --e) so.ustart[e] = u;
+          for (int e = t - 1; MULTI && e >= 0 && tabs[e].n == 0u; --e) so.ustart[e] = u;
         }
       }
       if (keep) {
@@ -432,6 +448,15 @@ __global__ void __launch_bounds__(SCAN_THREADS, GBA_SCAN_MINB)
       run[2] += __popc(nm);
       run[3] += __popc(nm & km);
     }
+  }
+  };
+  if constexpr (MULTI) {
+    if (mixed)
+      emit(std::true_type{});
+    else
+      emit(std::false_type{});
+  } else {
+    emit(std::false_type{});
   }
 }
 
