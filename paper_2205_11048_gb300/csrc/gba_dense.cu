@@ -237,6 +237,7 @@ __device__ __forceinline__ void st_hint(float4* a, float4 v, uint64_t policy) {
 __global__ void __launch_bounds__(256)
     k_dense_accumulate(float* __restrict__ hi, float* __restrict__ lo,
                        const float* __restrict__ g, int64_t D, float f, int first, int reverse) {
+  chain_wait();
   const int64_t D4 = D & ~3ll;
   const int64_t n4 = D4 / 4;
   const uint64_t policy = evict_first_policy();
@@ -356,8 +357,8 @@ void launch_dense_accumulate(float* hi, float* lo, const float* g, int64_t D, fl
   int64_t grid = (D / 4 + 255) / 256;
   if (grid > (int64_t)num_sms * 8) grid = (int64_t)num_sms * 8;
   if (grid < 1) grid = 1;
-  k_dense_accumulate<<<(unsigned)grid, 256, 0, s>>>(hi, lo, g, D, f, first ? 1 : 0,
-                                                    reverse && D >= ACC_TURN ? 1 : 0);
+  launch_chained(0, k_dense_accumulate, (unsigned)grid, 256, 0, s, hi, lo, g, D, f, first ? 1 : 0,
+                 reverse && D >= ACC_TURN ? 1 : 0);
 }
 
 void launch_dense_eager(const DenseArgs& da, const float* hi, const float* lo, bool has_sum,

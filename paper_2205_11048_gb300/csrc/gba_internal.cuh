@@ -96,7 +96,8 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // microsecond off each gap (0.03M ids 61.7 -> 54.5 us a step, 0.85M 209.6 ->
 // 200.2); above CHAIN_MAX_N occurrences the waiting blocks' places on the SMs
 // are worth more than the gaps (5.2M and 131M: 0.7% slower), so those steps'
-// kernels start in the plain order.
+// kernels start in the plain order.  Pulls, the copies of pushes and push-time
+// dense sums, which come one after another, are always chained (N = 0).
 constexpr int64_t CHAIN_MAX_N = 1 << 21;
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");

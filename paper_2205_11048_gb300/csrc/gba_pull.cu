@@ -20,6 +20,7 @@ __global__ void __launch_bounds__(PULL_THREADS)
     k_pull_rows(const float* __restrict__ w, int64_t V, int d, int id_mode, uint64_t mod_magic,
                 const HashInfo* hinfo, const int64_t* __restrict__ ids, int64_t n,
                 float* __restrict__ out, int lg, ErrSink err) {
+  chain_wait();
   const int L = 1 << lg;
   const int lane = threadIdx.x & 31;
   const int l = lane & (L - 1);
@@ -75,11 +76,8 @@ void launch_pull_rows(const float* w, int64_t V, int d, int id_mode, uint64_t mo
   int64_t grid = (n + per_block - 1) / per_block;
   const int64_t cap = (int64_t)num_sms * 8;
   if (grid > cap) grid = cap;
-  if (vec)
-    k_pull_rows<true><<<(unsigned)grid, PULL_THREADS, 0, s>>>(w, V, d, id_mode, mod_magic, hinfo, ids, n, out, lg, err);
-  else
-    k_pull_rows<false><<<(unsigned)grid, PULL_THREADS, 0, s>>>(w, V, d, id_mode, mod_magic, hinfo,
-                                                               ids, n, out, lg, err);
+  launch_chained(0, vec ? k_pull_rows<true> : k_pull_rows<false>, (unsigned)grid, PULL_THREADS, 0, s, w,
+                 V, d, id_mode, mod_magic, hinfo, ids, n, out, lg, err);
 }
 
 }  // namespace gba

@@ -36,6 +36,7 @@ __device__ __forceinline__ void copy_piece(const char* src, char* dst, uint32_t 
 }
 
 __global__ void __launch_bounds__(COPY_THREADS) k_push_copy(const __grid_constant__ CopyList cl) {
+  chain_wait();
   int k = 0;
   while (k + 1 < cl.n && blockIdx.x >= cl.first[k + 1]) ++k;
   const uint64_t at = (uint64_t)(blockIdx.x - cl.first[k]) * COPY_CHUNK;
@@ -64,8 +65,7 @@ cudaError_t launch_push_copy(CopyList cl, cudaStream_t s) {
   }
   if (blocks == 0) return cudaSuccess;
   // the launch's own status, not the thread's last error, which may be another's
-  void* args[] = {&cl};
-  return cudaLaunchKernel((const void*)k_push_copy, dim3((unsigned)blocks), dim3(COPY_THREADS), args, 0, s);
+  return launch_chained(0, k_push_copy, (unsigned)blocks, COPY_THREADS, 0, s, cl);
 }
 
 }  // namespace gba
