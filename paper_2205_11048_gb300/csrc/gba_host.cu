@@ -131,7 +131,8 @@ struct gba_handle {
 
   size_t meta_bytes = 0;
   char* d_meta[SLOTS] = {};
-  char* h_meta[META_SLOTS] = {};
+  char* h_meta[META_SLOTS] = {};    // pinned, mapped
+  void* d_h_meta[META_SLOTS] = {};  // the same memory as the device sees it
   cudaEvent_t meta_ev[META_SLOTS] = {};
   int meta_slot = 0;
 
@@ -895,8 +896,9 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
     for (int b = 0; b < SLOTS; ++b)
       if (!dev_alloc((void**)&h->d_meta[b], h->meta_bytes)) return fail(GBA_E_OOM);
     for (int i = 0; i < META_SLOTS; ++i) {
-      if (cudaHostAlloc((void**)&h->h_meta[i], h->meta_bytes, cudaHostAllocDefault) !=
+      if (cudaHostAlloc((void**)&h->h_meta[i], h->meta_bytes, cudaHostAllocMapped) !=
               cudaSuccess ||
+          cudaHostGetDevicePointer(&h->d_h_meta[i], h->h_meta[i], 0) != cudaSuccess ||
           cudaEventCreateWithFlags(&h->meta_ev[i], cudaEventDisableTiming) != cudaSuccess)
         return fail(GBA_E_OOM);
     }
@@ -1050,7 +1052,7 @@ int32_t gba_try_apply(gba_handle* h) {
   h->meta_slot = (h->meta_slot + 1) % META_SLOTS;
   cudaEventSynchronize(h->meta_ev[slot]);
   char* hp = h->h_meta[slot];
-  const size_t Mx = (size_t)h->max_buf;
+  const size_t Mx = (size_t)M;  // at most max_buf, for which the buffers are sized
   size_t off = 0;
   auto section = [&](size_t bytes) {
     size_t o = off;
@@ -1104,8 +1106,8 @@ int32_t gba_try_apply(gba_handle* h) {
                            ts.bpow2 * (double)ts.desc.opt.beta2);
     tabs[t] = tb;
   }
-  GBA_CUDA(h, cudaMemcpyAsync(dmeta, hp, h->meta_bytes, cudaMemcpyHostToDevice, sorts));
-  cudaEventRecord(h->meta_ev[slot], sorts);
+  const bool by_kernel = off <= META_BY_KERNEL;  // K1 brings it along
+  if (!by_kernel) GBA_CUDA(h, cudaMemcpyAsync(dmeta, hp, off, cudaMemcpyHostToDevice, sorts));
 
   StepArgs a{};
   a.k = h->k;
@@ -1131,8 +1133,10 @@ int32_t gba_try_apply(gba_handle* h) {
   // ---- K1: message weights (Eq. (1)); clears the per-step scratch
   {
     Timed tm(h, GBA_K_WEIGHTS, sorts);
-    launch_weights(a, sc, h->d_stats, MAX_PASSES * MAX_RADIX, sorts);
+    launch_weights(a, sc, h->d_stats, MAX_PASSES * MAX_RADIX, h->d_h_meta[slot], dmeta,
+                   by_kernel ? off : 0, sorts);
   }
+  cudaEventRecord(h->meta_ev[slot], sorts);  // the staging block may be written again
   // ---- K5 on the side stream, concurrently with the sort and segment-sum.
   // It is forked after the histogram kernel has validated every id, so a step
   // that fails its id check leaves the dense parameters untouched too.

@@ -405,8 +405,11 @@ __device__ __forceinline__ int message_of(const uint32_t* off, int M, uint32_t& 
 }
 
 // ---- launch wrappers (defined in the kernel translation units) ---------------
+// meta_bytes (a multiple of 16, at most META_BY_KERNEL; 0: none) of the step's
+// description are brought from host_meta (mapped pinned memory) to dev_meta.
+constexpr size_t META_BY_KERNEL = 32 * 1024;
 void launch_weights(const StepArgs& a, StepScratch sc, DevStats* stats, int n_hist_words,
-                    cudaStream_t s);
+                    const void* host_meta, void* dev_meta, size_t meta_bytes, cudaStream_t s);
 
 // ---- the sort of the step's keys
 constexpr int MAX_PASSES = 4;

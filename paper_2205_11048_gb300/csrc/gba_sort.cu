@@ -76,11 +76,27 @@ __device__ __forceinline__ uint64_t row_of_id(const StepArgs& a, const TableInfo
 
 // ---------------------------------------------------------------------------
 // K1: message weights of Eq. (1), kept-message list, dense staleness counters;
-// also clears the per-step sort scratch.
+// also clears the per-step sort scratch, and brings the step's description from
+// the host: a description of up to META_BY_KERNEL bytes is read from pinned host
+// memory here, while the kernel before may still run, instead of by a copy of its
+// own in front (about 6 us of a small step, with the gaps around it).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_message_weights(StepArgs a, StepScratch sc,
-                                                         DevStats* st, int n_hist_words) {
+__global__ void __launch_bounds__(256)
+    k_message_weights(StepArgs a, StepScratch sc, DevStats* st, int n_hist_words,
+                      const uint4* host_meta, uint4* dev_meta, int n16) {
+  extern __shared__ uint4 s_meta[];
   const int tid = threadIdx.x;
+  for (int i = tid; i < n16; i += blockDim.x) {
+    uint4 v;  // volatile: the host rewrites this memory between steps
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(host_meta + i)
+                 : "memory");
+    s_meta[i] = v;
+  }
+  chain_wait();
+  for (int i = tid; i < n16; i += blockDim.x) dev_meta[i] = s_meta[i];
+  __syncthreads();  // the tokens are read back below
   for (int i = tid; i < n_hist_words; i += blockDim.x) sc.hist[i] = 0u;
   if (tid < MAX_PASSES) sc.tile_counter[tid] = 0u;
   if (tid == 0) *sc.step_err = 0u;
@@ -526,8 +542,10 @@ size_t sort_status_words(int64_t N, int radix) {
 }
 
 void launch_weights(const StepArgs& a, StepScratch sc, DevStats* stats, int n_hist_words,
-                    cudaStream_t s) {
-  k_message_weights<<<1, 256, 0, s>>>(a, sc, stats, n_hist_words);
+                    const void* host_meta, void* dev_meta, size_t meta_bytes, cudaStream_t s) {
+  launch_chained(a.N, k_message_weights, 1, 256, meta_bytes, s, a, sc, stats, n_hist_words,
+                 static_cast<const uint4*>(host_meta), static_cast<uint4*>(dev_meta),
+                 (int)(meta_bytes / 16));
 }
 
 void launch_sort_histogram(const StepArgs& a, const SortPlan& plan, uint32_t* hist,
