@@ -512,10 +512,7 @@ struct SegOut {
 // rows of at most SMALL_MAX by one lane group of k_row_long each, longer ones
 // in chunks.
 constexpr int LONG_ROW = 4;
-#ifndef GBA_SMALL_MAX
-#define GBA_SMALL_MAX 32
-#endif
-constexpr int SMALL_MAX = GBA_SMALL_MAX;
+constexpr int SMALL_MAX = 64;  // half of that in smaller ranges
 static_assert(SMALL_MAX < 256, "a small row's count shares a word with its table");
 #ifndef GBA_SCAN_TILE
 #define GBA_SCAN_TILE 2048

@@ -114,11 +114,11 @@ __device__ __forceinline__ float row_denominator(int mode, uint32_t c_all, uint3
 #ifndef GBA_LOOKBACK_SLEEP_NS
 #define GBA_LOOKBACK_SLEEP_NS 64
 #endif
-#ifndef GBA_SCAN_MINB
-#define GBA_SCAN_MINB 4
-#endif
-template <bool MULTI, bool CACHED, bool UNIT>
-__global__ void __launch_bounds__(SCAN_THREADS, GBA_SCAN_MINB)
+// BIG: four blocks per SM at 64 registers; a step whose tiles are resident with
+// three all the same (up to CHAIN_MAX_N positions) is faster with 80 registers
+// (0.85M positions: 185.2 -> 181.8 us a step; 131M with 80 registers: 1.2% slower).
+template <bool MULTI, bool CACHED, bool UNIT, bool BIG>
+__global__ void __launch_bounds__(SCAN_THREADS, BIG ? 4 : 3)
     k_seg_scan(StepArgs a, SegTable tb0, const SegTable* tabs_g, SegOut so,
                const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals, DevStats* st,
                ErrSink err, int64_t wait_ns) {
@@ -610,6 +610,12 @@ inline uint32_t chunk_entries(int64_t n, int L, int num_sms) {
   return (uint32_t)(per * G);
 }
 
+// The longest rows that one lane group of k_row_long takes alone, for a range of
+// n occurrences: while all rows fit the machine at once, short ones, so that the
+// longest does not decide (32 against 64: 188 us against 192 a step of 0.85M ids);
+// otherwise longer ones, which save merging (131M ids: 7.76 -> 7.64 ms).
+inline uint32_t small_limit(int64_t n) { return n > (1 << 23) ? SMALL_MAX : SMALL_MAX / 2; }
+
 // The table of row record u among tables [t0, t1).
 __device__ __forceinline__ int table_of_row(const uint32_t* ustart, int t0, int t1, uint32_t u) {
   int lo = t0, hi = t1;
@@ -665,7 +671,7 @@ struct RowRegs {
 template <int CH, int CPL, bool ADAM, bool MULTI, bool AHEAD>
 __global__ void __launch_bounds__(ROW_THREADS, (CH * CPL <= 4 && !AHEAD) ? 4 : (CPL <= 2 ? 3 : 2))
     k_row_apply(StepArgs a, SegTable tb0, const SegTable* tabs, int t0, int t1, uint32_t chunk,
-                SegOut so, DevStats* st, ErrSink err) {
+                uint32_t small_max, SegOut so, DevStats* st, ErrSink err) {
   __shared__ RowSlot s_slot[ROW_WARPS][32];
   __shared__ uint4 s_rec[ROW_WARPS][33];  // the next batch's records
   chain_wait();
@@ -724,8 +730,8 @@ __global__ void __launch_bounds__(ROW_THREADS, (CH * CPL <= 4 && !AHEAD) ? 4 : (
 #pragma unroll
     for (int e = 0; e < LONG_ROW; ++e)
       p[e] = is_short && (uint32_t)e < n ? so.kl[ks + e] : nullptr;
-    const bool is_small = n > (uint32_t)LONG_ROW && n <= (uint32_t)SMALL_MAX;
-    const bool is_long = n > (uint32_t)SMALL_MAX;
+    const bool is_small = n > (uint32_t)LONG_ROW && n <= small_max;
+    const bool is_long = n > small_max;
     const uint32_t sm = __ballot_sync(FULL, is_small), lm = __ballot_sync(FULL, is_long);
     uint32_t small_at = 0u, long_at = 0u, item_at = 0u, part_at = 0u;
     uint32_t nch = 0u, nparts = 0u;
@@ -1083,8 +1089,8 @@ void launch_apply_as(const StepArgs& a, const RowRange& r, const SegTable* tabs,
   const int64_t want = (r.n + ROW_WARPS * G - 1) / (ROW_WARPS * G);
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms * bps, want));
   launch_chained(a.N, k_row_apply<CH, CPL, ADAM, MULTI, AHEAD>, (unsigned)grid, ROW_THREADS, 0, s, a,
-                 r.first, tabs, r.t0, r.t1, chunk_entries(r.n, (int)(32 / G), num_sms), so, stats,
-                 err);
+                 r.first, tabs, r.t0, r.t1, chunk_entries(r.n, (int)(32 / G), num_sms),
+                 small_limit(r.n), so, stats, err);
 }
 
 template <int CH, int CPL, bool ADAM, bool MULTI>
@@ -1128,8 +1134,13 @@ template <bool MULTI, bool CACHED, bool UNIT>
 void launch_scan_as(const StepArgs& a, const SegTable& tb0, const SegTable* tabs, const SegOut& so,
                     const uint32_t* keys, const uint32_t* vals, DevStats* stats, ErrSink err,
                     int64_t wait_ns, size_t smem, cudaStream_t s) {
-  launch_chained(a.N, k_seg_scan<MULTI, CACHED, UNIT>, (unsigned)scan_tiles(a.N), SCAN_THREADS, smem, s,
-                 a, tb0, tabs, so, keys, vals, stats, err, wait_ns);
+  const unsigned tiles = (unsigned)scan_tiles(a.N);
+  if (a.N > CHAIN_MAX_N)
+    launch_chained(a.N, k_seg_scan<MULTI, CACHED, UNIT, true>, tiles, SCAN_THREADS, smem, s, a, tb0,
+                   tabs, so, keys, vals, stats, err, wait_ns);
+  else
+    launch_chained(a.N, k_seg_scan<MULTI, CACHED, UNIT, false>, tiles, SCAN_THREADS, smem, s, a, tb0,
+                   tabs, so, keys, vals, stats, err, wait_ns);
 }
 
 }  // namespace
