@@ -580,46 +580,59 @@ float message_weight(const gba_handle* h, int64_t k_apply, int64_t token) {
   return s < (int64_t)h->h_wtab.size() ? h->h_wtab[s] : 0.f;
 }
 
-// Whether a kernel on the handle's device may read p itself: memory of that
-// device, or managed.  (Host memory goes through the copy engine, which reads
-// it at the link's rate.)
-bool device_readable(const gba_handle* h, const void* p) {
+// Where a kernel on the handle's device can read p itself: memory of that
+// device, managed memory, or pinned host memory (host: through the link).
+// nullptr: only a copy can.
+const void* device_address(const gba_handle* h, const void* p, bool& host) {
+  host = false;
   cudaPointerAttributes at{};
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return nullptr;
   }
-  return (at.type == cudaMemoryTypeDevice && at.device == h->device) ||
-         at.type == cudaMemoryTypeManaged;
+  if ((at.type == cudaMemoryTypeDevice && at.device == h->device) ||
+      at.type == cudaMemoryTypeManaged)
+    return p;
+  host = at.type == cudaMemoryTypeHost;
+  return host ? at.devicePointer : nullptr;
+}
+bool device_readable(const gba_handle* h, const void* p) {
+  bool host = false;
+  return device_address(h, p, host) != nullptr && !host;
 }
 
 // The copies of one push: arrays that the device can read are gathered and
-// copied by one launch (flush), the others are enqueued one by one.
+// copied by one launch for those in device memory and one for those in pinned
+// host memory (flush), the others are enqueued one by one.
 struct PushCopies {
   gba_handle* h;
-  CopyList cl;
-  explicit PushCopies(gba_handle* h_) : h(h_) { cl.n = 0; }
+  CopyList cl[2];
+  explicit PushCopies(gba_handle* h_) : h(h_) { cl[0].n = cl[1].n = 0; }
   cudaError_t add(void* dst, const void* src, size_t bytes) {
     if (bytes == 0) return cudaSuccess;
-    if (!device_readable(h, src)) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, h->stream);
-    if (cl.n == COPY_MAX) {
+    bool host = false;
+    const void* from = device_address(h, src, host);
+    if (!from) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, h->stream);
+    CopyList& c = cl[host ? 1 : 0];
+    if (c.n == COPY_MAX) {
       const cudaError_t e = flush();
       if (e != cudaSuccess) return e;
     }
-    cl.src[cl.n] = src;
-    cl.dst[cl.n] = dst;
-    cl.bytes[cl.n++] = bytes;
+    c.src[c.n] = from;
+    c.dst[c.n] = dst;
+    c.bytes[c.n++] = bytes;
     return cudaSuccess;
   }
   cudaError_t flush() {
-    if (cl.n == 0) return cudaSuccess;
+    if (cl[0].n == 0 && cl[1].n == 0) return cudaSuccess;
     // a launch needs the stream's device current; a copy did not
     int dev = h->device;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess && dev != h->device) e = cudaSetDevice(h->device);
-    if (e == cudaSuccess) e = launch_push_copy(cl, h->stream);
+    if (e == cudaSuccess && cl[0].n > 0) e = launch_push_copy(cl[0], 0xFFFFFFFFu, h->stream);
+    if (e == cudaSuccess && cl[1].n > 0) e = launch_push_copy(cl[1], HOST_BLOCKS, h->stream);
     if (dev != h->device) cudaSetDevice(dev);
-    cl.n = 0;
+    cl[0].n = cl[1].n = 0;
     return e;
   }
 };

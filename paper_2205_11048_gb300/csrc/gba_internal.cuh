@@ -562,10 +562,13 @@ struct CopyList {
   const void* src[COPY_MAX];
   void* dst[COPY_MAX];
   uint64_t bytes[COPY_MAX];
-  uint32_t first[COPY_MAX];  // first block of each array (set by launch_push_copy)
+  uint32_t first[COPY_MAX];  // first chunk of each array (set by launch_push_copy)
+  uint32_t chunks;           // chunks of them all (set by launch_push_copy)
   int32_t n;
 };
-cudaError_t launch_push_copy(CopyList cl, cudaStream_t s);
+// By at most max_blocks blocks.
+constexpr unsigned HOST_BLOCKS = 64;  // fill the link to host memory
+cudaError_t launch_push_copy(CopyList cl, unsigned max_blocks, cudaStream_t s);
 
 // Eager dense aggregation: add f * g to a step's accumulator (first: start it;
 // reverse: from the last parameter down), and the step's update from the
