@@ -13,6 +13,8 @@
 // mbarrier, and finish the tile with the optimizer.  Every mbarrier wait is
 // bounded in time; a wait that gives up latches ERR_TIMEOUT, the CTA stops
 // issuing copies, waits (bounded) for the copies it already issued, and exits.
+#include <algorithm>
+
 #include "gba_internal.cuh"
 
 namespace gba {
@@ -22,17 +24,21 @@ namespace {
 #ifndef GBA_DENSE_TILE
 #define GBA_DENSE_TILE 2048
 #endif
-#ifndef GBA_DENSE_STAGES
-#define GBA_DENSE_STAGES 8
-#endif
 constexpr int DT = GBA_DENSE_TILE;       // parameters per tile
-constexpr int STAGES = GBA_DENSE_STAGES;  // DT floats each
+// Stages of DT floats: as many as help the largest updates, or fewer, so that
+// three CTAs leave the kernels of the other streams 107 KB of an SM's shared memory
+// instead of 33, for updates that are short beside them (D x M of at most
+// DENSE_SHORT bytes, and more than one CTA per SM): steps of 1M x 32 gradients 186.1 ->
+// 178.2 us, 2M x 32 305.8 -> 295.8; with 5 stages 64M x 16 took 1% longer.
+constexpr int STAGES_LONG = 8, STAGES_SHORT = 5;
+constexpr int64_t DENSE_SHORT = 256ll << 20;
 constexpr int CONSUMER_WARPS = 8;        // 256 threads
 constexpr int HALF = CONSUMER_WARPS * 32 * 4;  // floats of one float4 per consumer thread
 constexpr int PER = DT / HALF;  // thread c owns [h*HALF + 4c, h*HALF + 4c + 4), h < PER
 static_assert(DT % HALF == 0, "a tile is a whole number of float4 rows of the consumers");
 constexpr int DENSE_THREADS = (CONSUMER_WARPS + 1) * 32;
 
+template <int STAGES>
 __global__ void __launch_bounds__(DENSE_THREADS)
     k_dense_apply(StepArgs a, DenseArgs da, StepScratch sc, ErrSink err, int64_t wait_ns) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -327,29 +333,48 @@ __global__ void __launch_bounds__(256)
 
 }  // namespace
 
-size_t dense_smem_bytes() { return (size_t)STAGES * DT * sizeof(float) + 2 * STAGES * sizeof(uint64_t); }
+namespace {
+
+template <int STAGES>
+constexpr size_t dense_smem() {
+  return (size_t)STAGES * DT * sizeof(float) + 2 * STAGES * sizeof(uint64_t);
+}
+
+template <int STAGES>
+void dense_as(const StepArgs& a, const DenseArgs& da, StepScratch sc, ErrSink err,
+              int64_t wait_ns, int num_sms, int64_t n_tiles, cudaStream_t s) {
+  constexpr size_t smem = dense_smem<STAGES>();
+  static const int bps = [&]() {  // persistent: as many CTAs as fit on an SM, at most three
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_dense_apply<STAGES>, DENSE_THREADS,
+                                                      smem) != cudaSuccess ||
+        b < 1)
+      b = 1;
+    return std::min(b, 3);
+  }();
+  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms * bps, n_tiles));
+  k_dense_apply<STAGES><<<(unsigned)grid, DENSE_THREADS, smem, s>>>(a, da, sc, err, wait_ns);
+}
+
+}  // namespace
 
 cudaError_t configure_dense() {
-  return cudaFuncSetAttribute(k_dense_apply, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)dense_smem_bytes());
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_dense_apply<STAGES_LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)dense_smem<STAGES_LONG>());
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_dense_apply<STAGES_SHORT>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)dense_smem<STAGES_SHORT>());
 }
 
 void launch_dense(const StepArgs& a, const DenseArgs& da, StepScratch sc, ErrSink err,
                   int64_t wait_ns, int num_sms, cudaStream_t s) {
-  const size_t smem = dense_smem_bytes();
   const int64_t n_tiles = ((da.D & ~3ll) + DT - 1) / DT;
-  static const int bps = [&]() {  // persistent: as many CTAs as fit on an SM
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_dense_apply, DENSE_THREADS, smem) !=
-            cudaSuccess ||
-        b < 1)
-      b = 1;
-    return b;
-  }();
-  int64_t grid = (int64_t)num_sms * bps;
-  if (grid > n_tiles) grid = n_tiles;
-  if (grid < 1) grid = 1;
-  k_dense_apply<<<(unsigned)grid, DENSE_THREADS, smem, s>>>(a, da, sc, err, wait_ns);
+  if (n_tiles > num_sms && da.D * 4 * da.M <= DENSE_SHORT)
+    dense_as<STAGES_SHORT>(a, da, sc, err, wait_ns, num_sms, n_tiles, s);
+  else
+    dense_as<STAGES_LONG>(a, da, sc, err, wait_ns, num_sms, n_tiles, s);
 }
 
 void launch_dense_accumulate(float* hi, float* lo, const float* g, int64_t D, float f, bool first,

@@ -550,7 +550,6 @@ struct DenseArgs {
                          // consumer wait runs out and reports ERR_TIMEOUT
 };
 
-size_t dense_smem_bytes();
 cudaError_t configure_dense();
 void launch_dense(const StepArgs& a, const DenseArgs& da, StepScratch sc, ErrSink err,
                   int64_t wait_ns, int num_sms, cudaStream_t s);

@@ -799,7 +799,7 @@ def test_copying_push_of_any_alignment(where, shift, eager):
         assert torch.equal(a, b)
 
 
-@pytest.mark.parametrize("D", [1, 3, 5, 8_000_003, 9_000_000])
+@pytest.mark.parametrize("D", [1, 3, 5, 8_000_003, 9_000_000, 17_000_003])
 def test_eager_dense_sizes(D):
     """Push-time sums equal the buffered ones bit for bit at the edges of the
     accumulate kernel: less than one float4, a ragged end, and sizes where the
