@@ -129,9 +129,11 @@ __global__ void __launch_bounds__(SCAN_THREADS, BIG ? 4 : 3)
   __shared__ uint32_t s_tile;
 
   chain_wait();
-  // block-uniform: another kernel may set the word while this block reads it
-  if (__syncthreads_or((ld_volatile_u32(err.step) & (ERR_ID_RANGE | ERR_TIMEOUT)) != 0u)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the step's state, the tile's ticket (by the last warp, which has the least to
+  // cache) and the lookups in flight together
+  const uint32_t failed = ld_volatile_u32(err.step) & (ERR_ID_RANGE | ERR_TIMEOUT);
+  if (tid == SCAN_THREADS - 1) s_tile = atomicAdd(so.ticket, 1u);
   const uint32_t lt = lanemask_lt();
   const int M = a.M, T = MULTI ? a.T : 1;
   const uint32_t* off_all = a.msg_off;            // [T][M + 1]
@@ -156,8 +158,8 @@ __global__ void __launch_bounds__(SCAN_THREADS, BIG ? 4 : 3)
     tok32 = c_tok;
     tabs = c_tabs;
   }
-  if (tid == 0) s_tile = atomicAdd(so.ticket, 1u);
-  __syncthreads();
+  // block-uniform: another kernel may set the word while this block reads it
+  if (__syncthreads_or(failed != 0u)) return;
   const uint32_t tile = s_tile;
   const uint32_t N = (uint32_t)a.N;  // below 2^30
   const uint32_t n_tiles = (N + SCAN_TILE - 1) / SCAN_TILE;
@@ -676,9 +678,10 @@ __global__ void __launch_bounds__(ROW_THREADS, (CH * CPL <= 4 && !AHEAD) ? 4 : (
   __shared__ uint4 s_rec[ROW_WARPS][33];  // the next batch's records
   chain_wait();
   // a failed step changes no row (warp-uniform: the warp reduces at the end)
-  if (__any_sync(FULL, ld_volatile_u32(err.step) != 0u)) return;
-  constexpr int P = CH * CPL;
+  const uint32_t failed = ld_volatile_u32(err.step);
   const uint32_t us = ld_volatile_u32(so.ustart + t0), ue = ld_volatile_u32(so.ustart + t1);
+  if (__any_sync(FULL, failed != 0u)) return;
+  constexpr int P = CH * CPL;
   const int d = tb0.d;
   const int C = CH == 4 ? d / 4 : d;  // pieces per row
   const int L = row_lanes(C, CPL);
@@ -908,7 +911,9 @@ __global__ void __launch_bounds__(ROW_THREADS, 2)
     k_row_long(StepArgs a, SegTable tb0, const SegTable* tabs, int t0, int t1, uint32_t chunk,
                SegOut so, DevStats* st, ErrSink err) {
   chain_wait();
-  if (__any_sync(FULL, ld_volatile_u32(err.step) != 0u)) return;
+  const uint32_t failed = ld_volatile_u32(err.step);
+  const uint32_t n_items = ld_volatile_u32(so.n_items), n_small = ld_volatile_u32(so.n_small);
+  if (__any_sync(FULL, failed != 0u)) return;
   constexpr int P = CH * CPL;
   constexpr int UNR = P <= 4 ? 8 : 4;
   const int d = tb0.d;
@@ -921,6 +926,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 2)
   const bool unit = a.decay == 0;  // every kept weight is 1
   const int32_t tag = (int32_t)(a.k + 1);
   uint32_t applied = 0u;
+  const uint32_t gw = blockIdx.x * (uint32_t)ROW_WARPS + (threadIdx.x >> 5);
+  const uint32_t W = gridDim.x * (uint32_t)ROW_WARPS;
   auto claim = [&](uint32_t* ticket, uint32_t n) {
     uint32_t v = 0u;
     if (lane == 0) v = atomicAdd(ticket, n);
@@ -941,12 +948,13 @@ __global__ void __launch_bounds__(ROW_THREADS, 2)
   // ---- 1. chunks of the longest rows, one warp per chunk; the warp's next
   // item is claimed and read while the current one is summed
   {
-    const uint32_t n_items = ld_volatile_u32(so.n_items);
-    uint32_t it = n_items ? claim(so.item_ticket, 1u) : 0u;
+    // a warp's first item is the one of its own number, the others are claimed
+    // behind those
+    uint32_t it = gw;
     uint2 item = it < n_items ? so.items[it] : make_uint2(0u, 0u);
     uint4 lr = it < n_items ? so.long_rows[item.x] : make_uint4(0u, 0u, 0u, 0u);
     while (it < n_items) {
-      const uint32_t it_next = claim(so.item_ticket, 1u);
+      const uint32_t it_next = W + claim(so.item_ticket, 1u);
       const uint2 item_next = it_next < n_items ? so.items[it_next] : make_uint2(0u, 0u);
       const uint32_t nch = (lr.z + chunk - 1) / chunk;
       const uint32_t e0 = lr.y + item.y * chunk;
@@ -1028,7 +1036,6 @@ __global__ void __launch_bounds__(ROW_THREADS, 2)
 
   // ---- 2. rows of LONG_ROW + 1 .. SMALL_MAX kept occurrences, one lane group each
   {
-    const uint32_t n_small = ld_volatile_u32(so.n_small);
     uint32_t base = n_small ? claim(so.small_ticket, (uint32_t)G) : 0u;
     uint4 sr = base + g < n_small ? so.small_rows[base + g] : make_uint4(0u, 0u, 0u, 0u);
     while (base < n_small) {

@@ -288,15 +288,17 @@ __global__ void __launch_bounds__(SORT_THREADS, ITEMS == 8 ? 5 : 4)
   if (FIRST)
     for (int i = tid; i < SORT_WARPS * RADIX; i += SORT_THREADS) s_kv[i] = 0u;
   chain_wait();
-  // An id range error was latched before this launch (by the histogram):
-  // every tile of every pass skips, consistently.
-  if (__syncthreads_or((ld_volatile_u32(err.step) & ERR_ID_RANGE) != 0u)) return;
-
-  if (tid == 0) s_tile = atomicAdd(sp.ticket, 1u);
+  // the tile's ticket, the step's state and its digit counts in flight together
+  uint32_t ticket = 0u;
+  if (tid == 0) ticket = atomicAdd(sp.ticket, 1u);
+  const uint32_t failed = ld_volatile_u32(err.step) & ERR_ID_RANGE;
   uint32_t hist_d[DPT];
 #pragma unroll
   for (int q = 0; q < DPT; ++q) hist_d[q] = sp.hist[tid * DPT + q];
-  __syncthreads();
+  if (tid == 0) s_tile = ticket;
+  // An id range error was latched before this launch (by the histogram):
+  // every tile of every pass skips, consistently.
+  if (__syncthreads_or(failed != 0u)) return;
 
   const uint32_t tile = s_tile, N = sp.N;
   const uint32_t base = tile * (uint32_t)TILE;
