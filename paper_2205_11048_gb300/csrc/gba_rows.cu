@@ -991,7 +991,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 2)
           for (int i = 0; i < P; ++i) acc[i] = CSum{0.f, 0.f};
           const uint32_t share = (nch + G - 1) / G;
           const uint32_t c0 = min(g * share, nch), c1 = min(c0 + share, nch);
-          constexpr int MU = P <= 4 ? 4 : 1;
+          constexpr int MU = P > 4 ? 1 : (CH == 4 ? 2 : 4);  // chunk sums in flight
           for (uint32_t cc = c0; cc < c1; cc += MU) {
             Part<CH, CPL> hi[MU], lo[MU];
 #pragma unroll
