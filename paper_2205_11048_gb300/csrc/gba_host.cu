@@ -1,6 +1,7 @@
 // Host side of libgba: the gradient buffer (FIFO of messages and the device
 // buffers their data live in), the assembly of a global step, kernel launches
 // on the handle's stream, error latching and the C ABI of include/gba.h.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -82,10 +83,6 @@ struct PendingTiming {
 size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
 }  // namespace
-
-#ifndef GBA_STREAM_PRIO
-#define GBA_STREAM_PRIO 0
-#endif
 
 struct gba_handle {
   int device = 0;
@@ -580,25 +577,50 @@ float message_weight(const gba_handle* h, int64_t k_apply, int64_t token) {
   return s < (int64_t)h->h_wtab.size() ? h->h_wtab[s] : 0.f;
 }
 
-// Where a kernel on the handle's device can read p itself: memory of that
-// device, managed memory, or pinned host memory (host: through the link).
-// nullptr: only a copy can.
-const void* device_address(const gba_handle* h, const void* p, bool& host) {
-  host = false;
-  cudaPointerAttributes at{};
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  if ((at.type == cudaMemoryTypeDevice && at.device == h->device) ||
-      at.type == cudaMemoryTypeManaged)
-    return p;
-  host = at.type == cudaMemoryTypeHost;
-  return host ? at.devicePointer : nullptr;
+// cuPointerGetAttributes, looked up once (the library does not link the driver).
+using PointerAttributesFn = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+PointerAttributesFn pointer_attributes() {
+  static const PointerAttributesFn fn = []() -> PointerAttributesFn {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault,
+                                         &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    return reinterpret_cast<PointerAttributesFn>(f);
+  }();
+  return fn;
 }
-bool device_readable(const gba_handle* h, const void* p) {
+
+// Where a kernel on the handle's device can read [p, p + bytes) itself: memory
+// of that device, managed memory, or pinned host memory (host: through the
+// link).  nullptr: only a copy can, or the range leaves its allocation, which
+// the copy refuses with an error where a kernel would fault.
+const void* device_address(const gba_handle* h, const void* p, size_t bytes, bool& host) {
+  host = false;
+  const PointerAttributesFn fn = pointer_attributes();
+  if (!fn) return nullptr;
+  unsigned int type = 0, managed = 0;
+  int device = -1;
+  CUdeviceptr at = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[] = {
+      CU_POINTER_ATTRIBUTE_MEMORY_TYPE,      CU_POINTER_ATTRIBUTE_IS_MANAGED,
+      CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,   CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+      CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* to[] = {&type, &managed, &device, &at, &start, &size};
+  if (fn(6, what, to, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS || at == 0) return nullptr;
+  const CUdeviceptr first = (CUdeviceptr)(uintptr_t)p;
+  if (first < start || first - start > size || bytes > size - (size_t)(first - start)) return nullptr;
+  if (managed != 0 || (type == CU_MEMORYTYPE_DEVICE && device == h->device)) return p;
+  host = type == CU_MEMORYTYPE_HOST;
+  return host ? (const void*)(uintptr_t)at : nullptr;
+}
+bool device_readable(const gba_handle* h, const void* p, size_t bytes) {
   bool host = false;
-  return device_address(h, p, host) != nullptr && !host;
+  return device_address(h, p, bytes, host) != nullptr && !host;
 }
 
 // The copies of one push: arrays that the device can read are gathered and
@@ -611,7 +633,7 @@ struct PushCopies {
   cudaError_t add(void* dst, const void* src, size_t bytes) {
     if (bytes == 0) return cudaSuccess;
     bool host = false;
-    const void* from = device_address(h, src, host);
+    const void* from = device_address(h, src, bytes, host);
     if (!from) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, h->stream);
     CopyList& c = cl[host ? 1 : 0];
     if (c.n == COPY_MAX) {
@@ -741,7 +763,7 @@ gba_status push_common(gba_handle* h, int64_t token, const gba_sparse_grad* per_
     if (f > 0.f) {
       const float* src = dense_grad;
       // summed where it lies, if the kernel can read it there (aligned float4)
-      if (copy && !(((uintptr_t)dense_grad & 15u) == 0 && device_readable(h, dense_grad))) {
+      if (copy && !(((uintptr_t)dense_grad & 15u) == 0 && device_readable(h, dense_grad, (size_t)h->D * sizeof(float)))) {
         GBA_CUDA(h, cudaMemcpyAsync(h->d_stage_dense, dense_grad, h->D * sizeof(float),
                                     cudaMemcpyDefault, h->stream));
         src = h->d_stage_dense;
@@ -837,17 +859,9 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
       return fail(GBA_E_CUDA);
     h->own_stream = true;
   }
-  // Stream priorities (GBA_STREAM_PRIO): 0 all equal; 1 the row path first and
-  // the next step's sort last; 2 the row path first, the others equal.
-  int prio_lo = 0, prio_hi = 0;
-  if (GBA_STREAM_PRIO != 0 && cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi) != cudaSuccess)
-    prio_lo = prio_hi = 0;
-  const int p_rows = GBA_STREAM_PRIO != 0 ? prio_hi : 0;
-  const int p_sort = GBA_STREAM_PRIO == 1 ? prio_lo : (GBA_STREAM_PRIO == 2 ? (prio_lo + prio_hi) / 2 : 0);
-  const int p_side = GBA_STREAM_PRIO != 0 ? (prio_lo + prio_hi) / 2 : 0;
-  if (cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, p_side) != cudaSuccess ||
-      cudaStreamCreateWithPriority(&h->sorts, cudaStreamNonBlocking, p_sort) != cudaSuccess ||
-      cudaStreamCreateWithPriority(&h->applys, cudaStreamNonBlocking, p_rows) != cudaSuccess ||
+  if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&h->sorts, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&h->applys, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_pushes, cudaEventDisableTiming) != cudaSuccess)
     return fail(GBA_E_CUDA);
   for (int b = 0; b < SLOTS; ++b)
