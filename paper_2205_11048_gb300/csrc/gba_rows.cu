@@ -1154,17 +1154,19 @@ void launch_scan_as(const StepArgs& a, const SegTable& tb0, const SegTable* tabs
 
 int64_t scan_tiles(int64_t N) { return (N + SCAN_TILE - 1) / SCAN_TILE; }
 
+// Beside one per row, chunks are of at least 32 entries per lane group; full ones,
+// or those of a range with fewer than twice what the warps take at a time (twice
+// that after the last halving).
 int64_t long_items(int64_t n, int num_sms) {
-  // beside one per row: full chunks, or those of a step with few
-  return n / 128 + 4 * (int64_t)num_sms * LONG_WARPS + 1;
+  return std::min(n / 32, n / 128 + 4 * (int64_t)num_sms * LONG_WARPS) + 1;
 }
 
 int64_t long_parts(int64_t n, int d, int num_sms) {
   const int CPL = (d & 3) == 0 ? (d <= 128 ? 1 : 2) : (d <= 32 ? 1 : d <= 64 ? 2 : d <= 128 ? 4 : 8);
   const int L = row_lanes((d & 3) == 0 ? d / 4 : d, CPL);
-  // chunks of full size, or smaller ones in a step of at most twice the chunks
-  // that the warps take at a time (twice that after the last halving)
-  return 2 * (n / (32 / L * (L == 32 ? 128 : 64))) + 2 * 4 * (int64_t)num_sms * LONG_WARPS + 1;
+  const int64_t G = 32 / L;
+  return 2 * std::min(n / (32 * G), n / (G * (L == 32 ? 128 : 64)) +
+                                        4 * (int64_t)num_sms * LONG_WARPS) + 1;
 }
 
 void launch_seg_scan(const StepArgs& a, const SegTable& tb0, const SegTable* tabs,
