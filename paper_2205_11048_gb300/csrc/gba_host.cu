@@ -1254,7 +1254,7 @@ int32_t gba_try_apply(gba_handle* h) {
     for (int t0 = 0, t1; t0 < T; t0 = t1) {
       for (t1 = t0 + 1; t1 < T && tabs[t1].d == tabs[t0].d && tabs[t1].opt.kind == tabs[t0].opt.kind;)
         ++t1;
-      const RowRange r{t0, t1, nbase[t1] - nbase[t0], tabs[t0]};
+      const RowRange r{t0, t1, nbase[t1] - nbase[t0], h->overlap ? 1 : 32, tabs[t0]};
       if (r.n == 0) continue;
       uint32_t* counters = sc.seg_ticket + 8 * t0;
       so.n_long = counters + 1;

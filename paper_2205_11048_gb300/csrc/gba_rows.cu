@@ -1117,7 +1117,7 @@ void launch_rows_as(const StepArgs& a, const RowRange& r, const SegTable* tabs, 
     static const int bps = blocks_per_sm(k_row_long<CH, CPL, ADAM, MULTI>, ROW_THREADS, 0);
     const int64_t warps = r.n / ((LONG_ROW + 1) * G) + r.n / SMALL_MAX + 1;
     const int64_t grid = std::max<int64_t>(
-        1, std::min<int64_t>((int64_t)num_sms * bps, (warps + ROW_WARPS - 1) / ROW_WARPS));
+        1, std::min<int64_t>((int64_t)num_sms * std::min(bps, r.long_blocks), (warps + ROW_WARPS - 1) / ROW_WARPS));
     launch_chained(a.N, k_row_long<CH, CPL, ADAM, MULTI>, (unsigned)grid, ROW_THREADS, 0, s, a, r.first,
                    tabs, r.t0, r.t1, chunk_entries(r.n, (int)(32 / G), num_sms), so, stats, err);
   }
