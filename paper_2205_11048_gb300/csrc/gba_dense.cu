@@ -242,7 +242,7 @@ __device__ __forceinline__ void st_hint(float4* a, float4 v, uint64_t policy) {
 
 __global__ void __launch_bounds__(256)
     k_dense_accumulate(float* __restrict__ hi, float* __restrict__ lo,
-                       const float* __restrict__ g, int64_t D, float f, int first, int reverse) {
+                       const float* g, int64_t D, float f, int first, int reverse) {
   chain_wait();
   const int64_t D4 = D & ~3ll;
   const int64_t n4 = D4 / 4;

@@ -98,6 +98,10 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // are worth more than the gaps (5.2M and 131M: 0.7% slower), so those steps'
 // kernels start in the plain order.  Pulls, the copies of pushes and push-time
 // dense sums, which come one after another, are always chained (N = 0).
+// A block may thus be resident while the kernel before still writes, so memory that
+// any kernel writes (parameters, tags, descriptions, a caller's ids and gradients) is
+// not read-only for a chained kernel's life: it is read by ordinary loads after
+// chain_wait, never by __ldg or through const __restrict__ parameters.
 constexpr int64_t CHAIN_MAX_N = 1 << 21;
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -17,8 +17,8 @@ constexpr int PULL_THREADS = 256;
 
 template <bool VEC>
 __global__ void __launch_bounds__(PULL_THREADS)
-    k_pull_rows(const float* __restrict__ w, int64_t V, int d, int id_mode, uint64_t mod_magic,
-                const HashInfo* hinfo, const int64_t* __restrict__ ids, int64_t n,
+    k_pull_rows(const float* w, int64_t V, int d, int id_mode, uint64_t mod_magic,
+                const HashInfo* hinfo, const int64_t* ids, int64_t n,
                 float* __restrict__ out, int lg, ErrSink err) {
   chain_wait();
   const int L = 1 << lg;
@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(PULL_THREADS)
   const int64_t groups = (int64_t)gridDim.x * (PULL_THREADS >> lg);
   const int64_t g0 = ((int64_t)blockIdx.x * PULL_THREADS + threadIdx.x) >> lg;
   for (int64_t i = g0; i < n; i += groups) {
-    const int64_t id = __ldg(ids + i);
+    const int64_t id = ids[i];
     bool ok = true;
     uint64_t row;
     bool fresh = false;  // HASH: an id never seen gets its initial values
@@ -52,12 +52,12 @@ __global__ void __launch_bounds__(PULL_THREADS)
     if (VEC) {
       const int C = d >> 2;
       for (int q = l; q < C; q += L) {
-        float4 v = ok ? __ldg(reinterpret_cast<const float4*>(src) + q)
-                      : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 v = ok ? reinterpret_cast<const float4*>(src)[q]
+                            : make_float4(0.f, 0.f, 0.f, 0.f);
         reinterpret_cast<float4*>(dst)[q] = v;
       }
     } else {
-      for (int q = l; q < d; q += L) dst[q] = ok ? __ldg(src + q) : 0.f;
+      for (int q = l; q < d; q += L) dst[q] = ok ? src[q] : 0.f;
     }
   }
 }

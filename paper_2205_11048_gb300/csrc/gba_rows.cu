@@ -120,8 +120,7 @@ __device__ __forceinline__ float row_denominator(int mode, uint32_t c_all, uint3
 template <bool MULTI, bool CACHED, bool UNIT, bool BIG>
 __global__ void __launch_bounds__(SCAN_THREADS, BIG ? 4 : 3)
     k_seg_scan(StepArgs a, SegTable tb0, const SegTable* tabs_g, SegOut so,
-               const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals, DevStats* st,
-               ErrSink err, int64_t wait_ns) {
+               const uint32_t* keys, const uint32_t* vals, DevStats* st, ErrSink err, int64_t wait_ns) {
   extern __shared__ __align__(16) unsigned char s_cache[];
   __shared__ uint32_t s_wsum[4][SCAN_WARPS];
   __shared__ uint32_t s_base[4];
@@ -219,7 +218,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, BIG ? 4 : 3)
         if (key[j] != NO_KEY) {
           if (MIX) t = advance(t, key[j]);
           const uint32_t x = key[j] - (MIX ? tabs[t] : tb1).key_base;
-          if (a.row_staleness == 0 && x < (MIX ? tabs[t] : tb1).rows) tg[j] = __ldg((MIX ? tabs[t] : tb1).ver + x);
+          if (a.row_staleness == 0 && x < (MIX ? tabs[t] : tb1).rows) tg[j] = (MIX ? tabs[t] : tb1).ver[x];
         }
       }
     }
@@ -623,7 +622,7 @@ __device__ __forceinline__ int table_of_row(const uint32_t* ustart, int t0, int 
   int lo = t0, hi = t1;
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
-    if (__ldg(ustart + mid) <= u)
+    if (ustart[mid] <= u)
       lo = mid;
     else
       hi = mid;

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
   __syncthreads();
   const uint32_t* offs = offs_cached ? s_off : a.msg_off;
   const uint32_t N = (uint32_t)a.N;  // below 2^30
-  auto first_of = [&](int t) { return tabs_cached ? s_nb[t] : (uint32_t)__ldg(a.nbase + t); };
+  auto first_of = [&](int t) { return tabs_cached ? s_nb[t] : (uint32_t)a.nbase[t]; };
   const uint32_t step = (uint32_t)(SORT_THREADS * HIST_ITEMS);
   auto table_at = [&](uint32_t o) {  // the last table that starts at or before o
     int lo = 0, hi = T;
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
 #pragma unroll
       for (int e = 0; e < HIST_ITEMS; ++e) {
         const uint32_t i = (uint32_t)(e * SORT_THREADS + tid);
-        if (i < here) id[e] = __ldg(src + i);
+        if (i < here) id[e] = src[i];
       }
       const TableInfo ti = a.tinfo[t1];
 #pragma unroll
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(SORT_THREADS)
         uint32_t x = base + i - first_of(t);
         const int m = message_at(t, x);
         tab[e] = t;
-        id[e] = __ldg(a.ids_ptr[(size_t)t * M + m] + x);
+        id[e] = a.ids_ptr[(size_t)t * M + m][x];
       }
 #pragma unroll
       for (int e = 0; e < HIST_ITEMS; ++e)
