@@ -208,6 +208,7 @@ gba_status set_err(gba_handle* h, gba_status s, const std::string& msg) {
 gba_status cuda_fail(gba_handle* h, cudaError_t e, const char* what) {
   std::string m = std::string(what) + ": " + cudaGetErrorString(e);
   if (h) h->last_error = m;
+  cudaGetLastError();  // reported here: the next step's launch check must not find it again
   return e == cudaErrorMemoryAllocation ? GBA_E_OOM : GBA_E_CUDA;
 }
 
@@ -704,22 +705,19 @@ gba_status push_common(gba_handle* h, int64_t token, const gba_sparse_grad* per_
   m.rows.resize(h->T);
   m.n.resize(h->T);
   m.arena_v.assign(h->T, -1);
-  if (copy) {
+  m.dense = nullptr;
+  std::vector<int64_t> saved_tail;  // of the arenas
+  auto store_copy = [&]() -> gba_status {
     gba_status s = ensure_arenas(h);
     if (s != GBA_OK) return s;
     // The copy may overwrite buffer space of messages that earlier steps read.
     if (h->overlap) join_steps(h);
     if (h->D > 0 && !eager && h->slot_count >= h->max_buf)
       return set_err(h, GBA_E_FULL, "gradient buffer full");
-    std::vector<int64_t> saved_tail(h->T);
-    for (int t = 0; t < h->T; ++t) saved_tail[t] = h->tables[t].arena.vtail;
+    for (const TableState& ts : h->tables) saved_tail.push_back(ts.arena.vtail);
     for (int t = 0; t < h->T; ++t) {
-      const int64_t n = per_table[t].n;
-      const int64_t v = h->tables[t].arena.alloc(n);
-      if (v < 0) {
-        for (int u = 0; u < h->T; ++u) h->tables[u].arena.vtail = saved_tail[u];
-        return set_err(h, GBA_E_FULL, "gradient buffer full (id storage)");
-      }
+      const int64_t v = h->tables[t].arena.alloc(per_table[t].n);
+      if (v < 0) return set_err(h, GBA_E_FULL, "gradient buffer full (id storage)");
       m.arena_v[t] = v;
     }
     PushCopies copies(h);
@@ -738,21 +736,13 @@ gba_status push_common(gba_handle* h, int64_t token, const gba_sparse_grad* per_
       const int32_t slot = (h->slot_head + h->slot_count) % h->max_buf;
       float* dst = h->dense_ring + (size_t)slot * h->D_pad;
       GBA_CUDA(h, copies.add(dst, dense_grad, h->D * sizeof(float)));
-      h->slot_count++;
       m.dense = dst;
-    } else {
-      m.dense = nullptr;
     }
     GBA_CUDA(h, copies.flush());
-  } else {
-    for (int t = 0; t < h->T; ++t) {
-      m.ids[t] = per_table[t].ids;
-      m.rows[t] = per_table[t].rows;
-      m.n[t] = per_table[t].n;
-    }
-    m.dense = dense_grad;
-  }
-  if (eager) {  // the dense gradient joins its step's accumulator now
+    return GBA_OK;
+  };
+  // eager: the dense gradient joins its step's accumulator now
+  auto accumulate = [&]() -> gba_status {
     if (new_group) {
       if (h->acc_ev_set[new_slot]) cudaStreamWaitEvent(h->stream, h->acc_ev[new_slot], 0);
       h->egroups.push_back(gba_handle::EagerGroup{0, new_slot, false, false});
@@ -779,8 +769,27 @@ gba_status push_common(gba_handle* h, int64_t token, const gba_sparse_grad* per_
       gr.reverse = !gr.reverse;
     }
     gr.accB += local_batch;
-    m.dense = nullptr;
+    return GBA_OK;
+  };
+  const size_t groups = h->egroups.size();
+  gba_status s = GBA_OK;
+  if (copy) {
+    s = store_copy();
+  } else {
+    for (int t = 0; t < h->T; ++t) {
+      m.ids[t] = per_table[t].ids;
+      m.rows[t] = per_table[t].rows;
+      m.n[t] = per_table[t].n;
+    }
+    if (!eager) m.dense = dense_grad;
   }
+  if (s == GBA_OK && eager) s = accumulate();
+  if (s != GBA_OK) {  // no message is stored, so nothing of the buffers is taken either
+    for (size_t t = 0; t < saved_tail.size(); ++t) h->tables[t].arena.vtail = saved_tail[t];
+    if (h->egroups.size() > groups) h->egroups.pop_back();
+    return s;
+  }
+  if (copy && m.dense) h->slot_count++;
   h->fifo.push_back(std::move(m));
   return GBA_OK;
 }
