@@ -499,7 +499,8 @@ gba_status grow_hash_tables(gba_handle* h, const std::vector<int64_t>& nbase) {
 gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
   if (N > h->n_cap) {
     sync_all(h);
-    int64_t cap = std::max<int64_t>(N + N / 4, 4096);
+    const int64_t cap = std::max<int64_t>(N + N / 4, 4096);
+    h->n_cap = 0;  // until every buffer is there: what a failed allocation leaves serves no step
     const size_t status_bytes = sort_status_words(cap, MAX_RADIX) * sizeof(unsigned long long);
     for (int b = 0; b < SLOTS; ++b) {
       for (int i = 0; i < 2; ++i) {
@@ -514,7 +515,6 @@ gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
       GBA_CUDA(h, cudaMalloc(&h->d_status[b], status_bytes));
       GBA_CUDA(h, cudaMemset(h->d_status[b], 0, status_bytes));
     }
-    h->n_cap = cap;
     // row-kernel buffers: a record per possible row (and one for the totals),
     // a kept-list entry per occurrence, look-back words per scan tile,
     // long rows and their chunks
@@ -547,6 +547,7 @@ gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
     GBA_CUDA(h, cudaMalloc(&h->d_items, (size_t)items_cap * sizeof(uint2)));
     GBA_CUDA(h, cudaMalloc(&h->d_part_hi, (size_t)part_floats * sizeof(float)));
     GBA_CUDA(h, cudaMalloc(&h->d_part_lo, (size_t)part_floats * sizeof(float)));
+    h->n_cap = cap;
   }
   return GBA_OK;
 }

@@ -100,3 +100,19 @@ def test_a_push_whose_copy_failed_takes_no_place_in_the_buffer(F, kind, nth, eag
     assert h.apply() == 1 and h.apply() == 0
     assert [h.push() for _ in range(4)] == [B.GBA_OK] * 3 + [B.GBA_E_FULL]
     assert h.apply() == 1
+
+
+@pytest.mark.parametrize("nth", range(1, 21))
+def test_a_step_whose_buffers_could_not_grow_is_refused_until_they_can(F, nth):
+    """The n-th of the step's allocations fails: the step is not applied and
+    stays buffered, a smaller one does not run on what is left of the buffers,
+    and the next that finds memory allocates all of them."""
+    h = Handle(F, G=1, max_buf=4, max_ids=200_000, dim=20)
+    assert h.push(n=600, ref=True) == B.GBA_OK
+    assert h.apply() == 1
+    assert h.push(n=100_000, ref=True) == B.GBA_OK and h.push(n=10, ref=True) == B.GBA_OK
+    for _ in range(2):
+        F.fake_fail(MALLOC, nth)
+        assert h.apply() == B.GBA_E_OOM
+    assert F.gba_pull_version(h.h) == 1
+    assert [h.apply(), h.apply(), h.apply()] == [1, 1, 0]
