@@ -11,6 +11,7 @@
 #include <deque>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "gba.h"
@@ -398,8 +399,7 @@ gba_status poll_device_error(gba_handle* h, bool force_sync) {
   return h->fail_code;
 }
 
-HashInfo hash_info(const gba_handle* h, int t) {
-  const TableState& ts = h->tables[t];
+HashInfo hash_info(const gba_handle* h, int t, const TableState& ts) {
   HashInfo hi{};
   hi.keys = ts.keys;
   hi.mask = (uint64_t)ts.desc.rows - 1;
@@ -425,7 +425,7 @@ gba_status layout_keys(gba_handle* h) {
     ts.key_base = (uint32_t)base;
     h->h_tinfo[t] = TableInfo{ts.desc.rows, (uint32_t)base, ts.desc.id_mode,
                               ~0ull / (uint64_t)ts.desc.rows};
-    h->h_hinfo[t] = ts.desc.id_mode == GBA_ID_HASH ? hash_info(h, t) : HashInfo{};
+    h->h_hinfo[t] = ts.desc.id_mode == GBA_ID_HASH ? hash_info(h, t, ts) : HashInfo{};
     base += (uint64_t)ts.desc.rows;
   }
   if (base >= 0xFFFFFFFFull) return set_err(h, GBA_E_ARG, "tables hold 2^32 - 1 rows or more");
@@ -456,44 +456,67 @@ gba_status alloc_hash_arrays(gba_handle* h, TableState& ts, uint64_t slots) {
   return GBA_OK;
 }
 
+// Moves a HASH table to `slots` slots, every id to its slot in the larger
+// table.  A table that cannot grow stays as it is.
+gba_status grow_hash_table(gba_handle* h, int t, uint64_t slots) {
+  TableState& ts = h->tables[t];
+  TableState grown = ts;
+  grown.w = grown.s0 = grown.s1 = nullptr;
+  grown.ver = nullptr;
+  grown.keys = nullptr;
+  grown.desc.rows = (int64_t)slots;
+  auto move_rows = [&]() -> gba_status {
+    const gba_status st = alloc_hash_arrays(h, grown, slots);
+    if (st != GBA_OK) return st;
+    launch_hash_rehash(hash_info(h, t, ts), hash_info(h, t, grown), h->stream);
+    GBA_CUDA(h, cudaGetLastError());
+    GBA_CUDA(h, cudaStreamSynchronize(h->stream));
+    return GBA_OK;
+  };
+  const gba_status st = move_rows();
+  if (st == GBA_OK) std::swap(ts, grown);
+  for (void* p : {(void*)grown.w, (void*)grown.s0, (void*)grown.s1, (void*)grown.ver,
+                  (void*)grown.keys})
+    cudaFree(p);
+  return st;
+}
+
 // Keeps every HASH table at most half full for the step about to run: the
 // bound on its ids grows by the step's occurrences; when it passes half the
 // slots the exact count is read, and if that is still too many the table
-// doubles until it is not, every id moving to its slot in the larger table.
+// doubles until it is not.  A step whose tables cannot grow is refused.
 gba_status grow_hash_tables(gba_handle* h, const std::vector<int64_t>& nbase) {
   bool changed = false;
-  for (int t = 0; t < h->T; ++t) {
+  gba_status st = GBA_OK;
+  for (int t = 0; t < h->T && st == GBA_OK; ++t) {
     TableState& ts = h->tables[t];
     if (ts.desc.id_mode != GBA_ID_HASH) continue;
     const int64_t Nt = nbase[t + 1] - nbase[t];
     ts.id_bound += Nt;
     if (ts.id_bound <= ts.desc.rows / 2) continue;
-    GBA_CUDA(h, sync_all(h));
     unsigned long long have = 0;
-    GBA_CUDA(h, cudaMemcpy(&have, ts.count, 8, cudaMemcpyDeviceToHost));
+    cudaError_t e = sync_all(h);
+    if (e == cudaSuccess) e = cudaMemcpy(&have, ts.count, 8, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) {
+      st = cuda_fail(h, e, "read a hash table's number of ids");
+      break;
+    }
     ts.id_bound = (int64_t)have + Nt;
     if (ts.id_bound <= ts.desc.rows / 2) continue;
     uint64_t slots = (uint64_t)ts.desc.rows;
     while ((int64_t)(slots / 2) < ts.id_bound) slots *= 2;
-    const HashInfo from = hash_info(h, t);
-    TableState old = ts;
-    ts.w = ts.s0 = ts.s1 = nullptr;
-    ts.ver = nullptr;
-    ts.keys = nullptr;
-    gba_status st = alloc_hash_arrays(h, ts, slots);
-    if (st != GBA_OK) return st;
-    ts.desc.rows = (int64_t)slots;
-    launch_hash_rehash(from, hash_info(h, t), h->stream);
-    GBA_CUDA(h, cudaGetLastError());
-    GBA_CUDA(h, cudaStreamSynchronize(h->stream));
-    cudaFree(old.w);
-    cudaFree(old.s0);
-    cudaFree(old.s1);
-    cudaFree(old.ver);
-    cudaFree(old.keys);
-    changed = true;
+    st = grow_hash_table(h, t, slots);
+    changed = changed || st == GBA_OK;
   }
-  return changed ? layout_keys(h) : GBA_OK;
+  if (changed) {  // also where a later table could not grow
+    const gba_status sl = layout_keys(h);
+    if (sl != GBA_OK) {
+      h->failed = true;
+      h->fail_code = sl;
+    }
+    if (st == GBA_OK) st = sl;
+  }
+  return st;
 }
 
 gba_status ensure_step_capacity(gba_handle* h, int64_t N) {

@@ -30,6 +30,12 @@ void launch_weights(const StepArgs&, StepScratch, DevStats*, int, const void*, v
 void launch_sort_histogram(const StepArgs& a, const SortPlan&, uint32_t*, uint32_t* keys0, ErrSink, int,
                            cudaStream_t) {
   fake_need(keys0, (size_t)a.N * 4);
+  for (int t = 0; t < a.T; ++t)  // the tables as the kernel would find them
+    if (a.tinfo[t].id_mode == 2) {
+      const HashInfo& h = a.hinfo[t];
+      fake_need(h.w, (size_t)a.tinfo[t].V * h.d * 4);
+      fake_need(h.keys, (size_t)(h.mask + 1) * 8);
+    }
 }
 void launch_onesweep(const SortPlan& plan, int, SortPass sp, ErrSink, int64_t, cudaStream_t) {
   for (const uint32_t* p : {sp.keys_in, (const uint32_t*)sp.keys_out, (const uint32_t*)sp.vals_out})

@@ -51,11 +51,12 @@ def _clean(F):
 class Handle:
     open = []
 
-    def __init__(self, F, dim=4, mode=0, G=3, max_buf=3, max_ids=8, D=8, rows=100, kind=0):
+    def __init__(self, F, dim=4, mode=0, G=3, max_buf=3, max_ids=8, D=8, rows=100, kind=0, more=None):
         self.F, self.dim, self.D = F, dim, D
         self.h = ctypes.c_void_p()
-        t = B.gba_table_desc(rows, dim, mode, max_ids, B.opt_desc(kind, 0.01))
-        assert F.gba_create((B.gba_table_desc * 1)(t), 1, D, ctypes.byref(B.opt_desc()), G, max_buf, None,
+        tables = [B.gba_table_desc(rows, dim, mode, max_ids, B.opt_desc(kind, 0.01))] + (more or [])
+        self.T = len(tables)
+        assert F.gba_create((B.gba_table_desc * self.T)(*tables), self.T, D, ctypes.byref(B.opt_desc()), G, max_buf, None,
                             0, None, ctypes.byref(self.h)) == B.GBA_OK
         Handle.open.append(self.h)
         self.keep = []
@@ -64,7 +65,7 @@ class Handle:
         ids, rows, dense = np.arange(n), np.zeros((n, self.dim), np.float32), np.zeros(self.D + 4, np.float32)
         at = (dense.ctypes.data + 15) & ~15
         self.keep.append((ids, rows, dense))
-        g = (B.gba_sparse_grad * 1)(B.gba_sparse_grad(ids.ctypes.data, n, rows.ctypes.data))
+        g = (B.gba_sparse_grad * self.T)(*[B.gba_sparse_grad(ids.ctypes.data, n, rows.ctypes.data)] * self.T)
         return (self.F.gba_push_ref if ref else self.F.gba_push)(self.h, 0, g, at, 1)
 
     def apply(self):
@@ -116,3 +117,34 @@ def test_a_step_whose_buffers_could_not_grow_is_refused_until_they_can(F, nth):
         assert h.apply() == B.GBA_E_OOM
     assert F.gba_pull_version(h.h) == 1
     assert [h.apply(), h.apply(), h.apply()] == [1, 1, 0]
+
+
+# four arrays, five with Adam's second moment
+@pytest.mark.parametrize("kind,nth", [(0, n) for n in range(1, 5)] + [(1, n) for n in range(1, 6)])
+def test_a_hash_table_that_could_not_grow_keeps_its_rows(F, kind, nth):
+    """The n-th of the larger table's allocations fails: the step is refused,
+    the table stays as it is, and a later step grows it."""
+    h = Handle(F, G=1, max_buf=4, max_ids=4096, rows=1024, mode=B.HASH, kind=kind)
+    assert h.push(n=400, ref=True) == B.GBA_OK
+    assert h.apply() == 1
+    before, n = h.arrays(), F.fake_allocations()
+    assert h.push(n=600, ref=True) == B.GBA_OK
+    for _ in range(2):
+        F.fake_fail(MALLOC, nth)
+        assert h.apply() == B.GBA_E_OOM
+        assert (h.arrays(), h.capacity(), F.fake_allocations()) == (before, 1024, n)
+    assert h.apply() == 1
+    assert h.capacity() == 2048
+
+
+@pytest.mark.parametrize("nth", range(5, 9))
+def test_the_second_of_two_hash_tables_could_not_grow(F, nth):
+    """The first table has grown when the second cannot: the steps that follow
+    find the first where it is now."""
+    h = Handle(F, G=1, max_buf=4, max_ids=4096, rows=1024, mode=B.HASH,
+               more=[B.gba_table_desc(1024, 4, B.HASH, 4096, B.opt_desc(0, 0.01))])
+    assert h.push(n=600, ref=True) == B.GBA_OK
+    F.fake_fail(MALLOC, nth)
+    assert h.apply() == B.GBA_E_OOM
+    assert h.capacity() == 2048
+    assert h.apply() == 1
