@@ -22,6 +22,8 @@ using namespace gba;
 namespace {
 
 constexpr int MAX_DIM = 256;
+constexpr uint64_t MAX_ROWS = 0xFFFFFFFFull;  // of all tables: keys are 32-bit, one value reserved
+constexpr const char* TOO_MANY_ROWS = "tables hold 2^32 - 1 rows or more";
 constexpr int MAX_DIGIT_BITS = 9;  // of a sort pass
 constexpr int MAX_RADIX = 1 << MAX_DIGIT_BITS;
 constexpr int META_SLOTS = 4;
@@ -428,7 +430,7 @@ gba_status layout_keys(gba_handle* h) {
     h->h_hinfo[t] = ts.desc.id_mode == GBA_ID_HASH ? hash_info(h, t, ts) : HashInfo{};
     base += (uint64_t)ts.desc.rows;
   }
-  if (base >= 0xFFFFFFFFull) return set_err(h, GBA_E_ARG, "tables hold 2^32 - 1 rows or more");
+  if (base >= MAX_ROWS) return set_err(h, GBA_E_ARG, TOO_MANY_ROWS);
   const uint64_t kmax = base > 0 ? base - 1 : 0;
   uint32_t bits = 1;
   while (bits < 32 && (kmax >> bits) != 0) ++bits;
@@ -505,7 +507,10 @@ gba_status grow_hash_tables(gba_handle* h, const std::vector<int64_t>& nbase) {
     if (ts.id_bound <= ts.desc.rows / 2) continue;
     uint64_t slots = (uint64_t)ts.desc.rows;
     while ((int64_t)(slots / 2) < ts.id_bound) slots *= 2;
-    st = grow_hash_table(h, t, slots);
+    uint64_t total = slots;  // of all tables, whose rows are the sort's 32-bit keys
+    for (int u = 0; u < h->T; ++u)
+      if (u != t) total += (uint64_t)h->tables[u].desc.rows;
+    st = total >= MAX_ROWS ? set_err(h, GBA_E_ARG, TOO_MANY_ROWS) : grow_hash_table(h, t, slots);
     changed = changed || st == GBA_OK;
   }
   if (changed) {  // also where a later table could not grow
@@ -848,7 +853,7 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
     }
     total_rows += r;
   }
-  if (total_rows >= 0xFFFFFFFFull) return GBA_E_ARG;  // keys are 32-bit, one value reserved
+  if (total_rows >= MAX_ROWS) return GBA_E_ARG;
   if (dense_size > 0 && validate_opt(*dense_opt) != GBA_OK) return GBA_E_ARG;
   gba_staleness_desc rule{0x7FFFFFFF, 0, 0, 0, 1.0f, 0};
   if (st) rule = *st;

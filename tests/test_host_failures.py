@@ -148,3 +148,16 @@ def test_the_second_of_two_hash_tables_could_not_grow(F, nth):
     assert h.apply() == B.GBA_E_OOM
     assert h.capacity() == 2048
     assert h.apply() == 1
+
+
+def test_a_hash_table_does_not_grow_past_the_keys(F):
+    """Growth that would bring the tables to 2^32 - 1 rows is refused before
+    anything changes: the table keeps its rows, and the handle is not failed."""
+    h = Handle(F, G=1, max_buf=4, max_ids=4096, rows=1024, mode=B.HASH, dim=1,
+               more=[B.gba_table_desc(2**32 - 2 - 1024, 1, B.DIRECT, 4096, B.opt_desc(0, 0.01))])
+    assert h.push(n=600, ref=True) == B.GBA_OK
+    before = h.arrays()
+    for _ in range(3):
+        assert h.apply() == B.GBA_E_ARG
+    assert (h.arrays(), h.capacity()) == (before, 1024)
+    assert F.gba_sync(h.h) == B.GBA_OK
