@@ -813,7 +813,9 @@ __global__ void __launch_bounds__(ROW_THREADS, (CH * CPL <= 4 && !AHEAD) ? 4 : (
 #pragma unroll
       for (int e = 0; e < P; ++e) {
         if (f0 == 1.f) {
-          acc[e] = CSum{r.g0.v[e], 0.f};  // 0 + g is exact: the first term as it is
+          // the first term as it is: 0 + g is exact, and its error g - g is 0, or NaN
+          // for an infinite g, as in the sums that start from zero
+          acc[e] = CSum{r.g0.v[e], __fsub_rn(r.g0.v[e], r.g0.v[e])};
         } else {
           acc[e] = CSum{0.f, 0.f};
           csum_add_prod(acc[e], f0, r.g0.v[e]);

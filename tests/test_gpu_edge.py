@@ -361,6 +361,53 @@ def test_chunk_boundaries_of_long_rows(dim, n):
     run_custom(cfg, [batch(0), batch(1), batch(2)], max_ids=sum(counts))
 
 
+@pytest.mark.parametrize("dim", [4, 7, 20, 70, 132])
+@pytest.mark.parametrize("rule", [dict(iota=1), dict(iota=1, decay=1, lam=0.5)])
+def test_non_finite_gradients_reach_their_elements_only(dim, rule):
+    """An infinite or NaN kept gradient makes its element's weight and state NaN
+    (the compensated sum of an infinity is NaN), whatever its place among the
+    row's occurrences and however many there are; the row's other elements are
+    those of finite gradients bit for bit, and a dropped one changes nothing."""
+    counts = [1, 1, 2, 4, 5, 31, 40, 700, 3]  # in the first message; the second lacks row 0
+    gen = torch.Generator(device="cuda").manual_seed(dim)
+    per = [torch.cat([torch.full((c,), r) for r, c in enumerate(counts) if r >= m]) for m in range(2)]
+    ids = [p.to("cuda", torch.int64) for p in per + [torch.tensor([len(counts) - 1])]]
+    rows = [torch.randn(i.numel(), dim, generator=gen, device="cuda") for i in ids]
+    dense = torch.zeros(4, device="cuda")
+    bad = [r.clone() for r in rows]
+    for r in range(len(counts) - 1):  # of the last row only a dropped occurrence is infinite
+        first, last = (ids[0] == r).nonzero()[0, 0], (ids[min(r, 1)] == r).nonzero()[-1, 0]
+        bad[0][first, 0] = float("inf")
+        bad[min(r, 1)][last, 1] = float("-inf")
+        bad[0][first, 2] = float("nan")
+    bad[2][0, 3] = float("inf")
+    torch.cuda.synchronize()
+    states = []
+    for grads in (rows, bad):
+        g = B.GBA([(len(counts), dim, 0, ids[0].numel(), B.opt_desc(0, 0.01))], 4, B.opt_desc(0, 0.01), 2, 4,
+                  seed=1, **rule)
+        for k in range(3):  # so that a token can be stale
+            for m in range(2):
+                g.push_ref(k, [ids[m]], [rows[m]], dense, 1)
+            assert g.try_apply() == 1
+        for m in range(2):
+            g.push_ref(3, [ids[m]], [grads[m]], dense, 1)
+        assert g.try_apply() == 1
+        g.push_ref(0, [ids[2]], [grads[2]], dense, 1)  # dropped: four steps old
+        g.push_ref(4, [ids[2][:0]], [rows[2][:0]], dense, 1)
+        assert g.try_apply() == 1
+        g.sync()
+        states.append([x.clone() for x in g.table(0)[:2]] + [g.table(0)[3].clone()])
+        g.close()
+    hit = torch.zeros(len(counts), dim, dtype=torch.bool, device="cuda")
+    hit[:-1, :3] = True
+    for fine, got in zip(states[0][:2], states[1][:2]):
+        assert torch.isfinite(fine).all()
+        assert torch.isnan(got[hit]).all()
+        assert torch.equal(got[~hit], fine[~hit])
+    assert torch.equal(states[0][2], states[1][2])
+
+
 def test_tables_that_share_launches():
     """Runs of tables of one width and optimizer, other widths and optimizers
     between them, and tables without ids first, last, between and alone in
