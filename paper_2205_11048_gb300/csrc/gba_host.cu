@@ -87,6 +87,9 @@ size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
 }  // namespace
 
+// Fresh buffers are cleared and descriptions copied on the handle's stream: the
+// kernels' streams do not wait for the default stream, where cudaMemset and
+// cudaMemcpy may still be under way when they return.
 struct gba_handle {
   int device = 0;
   int num_sms = 152;
@@ -436,10 +439,10 @@ gba_status layout_keys(gba_handle* h) {
   while (bits < 32 && (kmax >> bits) != 0) ++bits;
   h->plan = make_sort_plan((int)bits, MAX_DIGIT_BITS);
   if (h->T > 0) {
-    GBA_CUDA(h, cudaMemcpy(h->d_tinfo, h->h_tinfo.data(), h->T * sizeof(TableInfo),
-                           cudaMemcpyHostToDevice));
-    GBA_CUDA(h, cudaMemcpy(h->d_hinfo, h->h_hinfo.data(), h->T * sizeof(HashInfo),
-                           cudaMemcpyHostToDevice));
+    GBA_CUDA(h, cudaMemcpyAsync(h->d_tinfo, h->h_tinfo.data(), h->T * sizeof(TableInfo),
+                                cudaMemcpyHostToDevice, h->stream));
+    GBA_CUDA(h, cudaMemcpyAsync(h->d_hinfo, h->h_hinfo.data(), h->T * sizeof(HashInfo),
+                                cudaMemcpyHostToDevice, h->stream));
   }
   return GBA_OK;
 }
@@ -541,7 +544,7 @@ gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
       cudaFree(h->d_status[b]);
       h->d_status[b] = nullptr;
       GBA_CUDA(h, cudaMalloc(&h->d_status[b], status_bytes));
-      GBA_CUDA(h, cudaMemset(h->d_status[b], 0, status_bytes));
+      GBA_CUDA(h, cudaMemsetAsync(h->d_status[b], 0, status_bytes, h->stream));
     }
     // row-kernel buffers: a record per possible row (and one for the totals),
     // a kept-list entry per occurrence, look-back words per scan tile,
@@ -568,7 +571,8 @@ gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
     GBA_CUDA(h, cudaMalloc(&h->d_kl, (size_t)cap * sizeof(float*)));
     GBA_CUDA(h, cudaMalloc(&h->d_kw, (size_t)cap * sizeof(float)));
     GBA_CUDA(h, cudaMalloc(&h->d_scan_status, (size_t)stiles * 4 * sizeof(unsigned long long)));
-    GBA_CUDA(h, cudaMemset(h->d_scan_status, 0, (size_t)stiles * 4 * sizeof(unsigned long long)));
+    GBA_CUDA(h, cudaMemsetAsync(h->d_scan_status, 0, (size_t)stiles * 4 * sizeof(unsigned long long),
+                                h->stream));
     GBA_CUDA(h, cudaMalloc(&h->d_long_rows, (size_t)long_cap * sizeof(uint4)));
     GBA_CUDA(h, cudaMalloc(&h->d_small_rows, (size_t)long_cap * sizeof(uint4)));
     GBA_CUDA(h, cudaMalloc(&h->d_long_done, (size_t)long_cap * sizeof(uint32_t)));
@@ -591,7 +595,7 @@ gba_status ensure_arenas(gba_handle* h) {
   if (h->D > 0) {
     const size_t bytes = (size_t)h->max_buf * h->D_pad * sizeof(float);
     GBA_CUDA(h, cudaMalloc(&h->dense_ring, bytes));
-    GBA_CUDA(h, cudaMemset(h->dense_ring, 0, bytes));
+    GBA_CUDA(h, cudaMemsetAsync(h->dense_ring, 0, bytes, h->stream));
   }
   h->arenas_ready = true;
   return GBA_OK;
@@ -930,7 +934,8 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
     TableState& ts = h->tables[t];
     if (ts.desc.id_mode == GBA_ID_HASH) {
       if (alloc_hash_arrays(h, ts, (uint64_t)ts.desc.rows) != GBA_OK ||
-          !dev_alloc((void**)&ts.count, 8) || cudaMemset(ts.count, 0, 8) != cudaSuccess)
+          !dev_alloc((void**)&ts.count, 8) ||
+          cudaMemsetAsync(ts.count, 0, 8, h->stream) != cudaSuccess)
         return fail(GBA_E_OOM);
       continue;
     }
@@ -975,7 +980,7 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
                          align16((size_t)std::max(h->T, 1) * 32) + align16(M * 4);
     for (int b = 0; b < SLOTS; ++b) {
       if (!dev_alloc((void**)&h->d_step_scratch[b], bytes)) return fail(GBA_E_OOM);
-      if (cudaMemset(h->d_step_scratch[b], 0, bytes) != cudaSuccess) return fail(GBA_E_CUDA);
+      if (cudaMemsetAsync(h->d_step_scratch[b], 0, bytes, h->stream) != cudaSuccess) return fail(GBA_E_CUDA);
       char* p = h->d_step_scratch[b];
       StepScratch& sc = h->sc[b];
       sc.hist = (uint32_t*)p;
@@ -1006,8 +1011,8 @@ gba_status gba_create(const gba_table_desc* tables, int32_t n_tables, int64_t de
       pw = pw * (double)rule.lambda;
     }
     if (!dev_alloc((void**)&h->d_wtab, wt.size() * sizeof(float))) return fail(GBA_E_OOM);
-    if (cudaMemcpy(h->d_wtab, wt.data(), wt.size() * sizeof(float), cudaMemcpyHostToDevice) !=
-        cudaSuccess)
+    if (cudaMemcpyAsync(h->d_wtab, wt.data(), wt.size() * sizeof(float), cudaMemcpyHostToDevice,
+                        h->stream) != cudaSuccess)
       return fail(GBA_E_CUDA);
   }
   if (!dev_alloc((void**)&h->d_err, 4) || !dev_alloc((void**)&h->d_stats, sizeof(DevStats)))

@@ -15,7 +15,7 @@ namespace {
 enum { MALLOC = 0, MEMCPY_ASYNC = 1, PUSH_COPY = 2, KINDS = 3 };
 int g_fail[KINDS];    // the n-th call of the kind from now fails (0: none does)
 int g_addressable;    // arrays are device memory (copied by the launch) or unknown to the driver
-int g_bad;
+int g_bad, g_unordered;
 cudaError_t g_last = cudaSuccess;
 std::map<const char*, size_t>& live() {
   static std::map<const char*, size_t> m;
@@ -55,6 +55,7 @@ extern "C" {
 void fake_fail(int kind, int nth) { g_fail[kind] = nth; }
 void fake_addressable(int on) { g_addressable = on; }
 int fake_bad() { return g_bad; }
+int fake_unordered() { return g_unordered; }
 long fake_allocations() { return (long)live().size(); }
 cudaError_t fake_copy_launch() {
   return fails(PUSH_COPY) ? error(cudaErrorLaunchOutOfResources) : cudaSuccess;
@@ -75,14 +76,19 @@ cudaError_t cudaFree(void* p) { return release(p); }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned int) { return allocate(p, n); }
 cudaError_t cudaFreeHost(void* p) { return release(p); }
 cudaError_t cudaHostGetDevicePointer(void** d, void* p, unsigned int) { return *d = p, cudaSuccess; }
-cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
+// these use the default stream, on which the handle's streams do not wait
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind kind) {
+  if (kind != cudaMemcpyDeviceToHost) ++g_unordered;
   return memcpy(d, s, n), cudaSuccess;
+}
+cudaError_t cudaMemset(void* p, int v, size_t n) {
+  ++g_unordered;
+  return memset(p, v, n), cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
   if (fails(MEMCPY_ASYNC)) return error(cudaErrorInvalidValue);
   return memcpy(d, s, n), cudaSuccess;
 }
-cudaError_t cudaMemset(void* p, int v, size_t n) { return memset(p, v, n), cudaSuccess; }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) {
   return memset(p, v, n), cudaSuccess;
 }

@@ -161,3 +161,15 @@ def test_a_hash_table_does_not_grow_past_the_keys(F):
         assert h.apply() == B.GBA_E_ARG
     assert (h.arrays(), h.capacity()) == (before, 1024)
     assert F.gba_sync(h.h) == B.GBA_OK
+
+
+def test_fresh_buffers_are_filled_in_the_order_of_the_handles_streams(F):
+    """Nothing clears or fills device memory on the default stream: the first
+    copies of a push and the first kernels of a step do not wait for it, so a
+    clear still under way would take what they have written (a race, so it is
+    shown here and not on a GPU)."""
+    before = F.fake_unordered()
+    h = Handle(F, G=1, max_buf=4, max_ids=4096, rows=1024, mode=B.HASH)
+    assert [h.push(n=600), h.apply(), h.push(n=4000), h.apply()] == [B.GBA_OK, 1, B.GBA_OK, 1]
+    assert h.capacity() > 1024
+    assert F.fake_unordered() == before
