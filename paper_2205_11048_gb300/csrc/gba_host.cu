@@ -33,6 +33,12 @@ constexpr int EAGER_SLOTS = 8;  // pending global steps with eager dense accumul
 // Per-step buffers exist twice, so that step k + 1's message weights and sort
 // run (on the sort stream) while step k's segment-sum and dense update run.
 constexpr int SLOTS = 2;
+// A step's buffers of more than so many bytes are one allocation; up to there an
+// allocation each, which find room beside earlier ones where one of the whole size
+// is mapped anew.  First step of a handle, always apart -> as it is: 30,000 ids x 24
+// floats 285 -> 203 us, 100,000 x 128 485 -> 240, 0.4M x 64 810 -> 278.  Always in
+// one: 6,000 ids in three tables 160 -> 215, 4,347 x 208 142 -> 198.
+constexpr size_t ONE_STEP_BLOCK = 5 << 19;
 
 struct Arena {  // contiguous-allocation ring over [0, cap) with virtual offsets
   int64_t cap = 0;
@@ -139,8 +145,10 @@ struct gba_handle {
   cudaEvent_t meta_ev[META_SLOTS] = {};
   int meta_slot = 0;
 
-  // sort / segment scratch, grown on demand
+  // sort / segment scratch, grown on demand: the allocations that hold the arrays below
+  std::vector<char*> step_blocks;
   int64_t n_cap = 0;
+  int32_t cap_radix = 0;  // the sort's counters per pass it is sized for
   uint32_t* d_keys[SLOTS][2] = {};
   uint32_t* d_vals[SLOTS][2] = {};
   unsigned long long* d_status[SLOTS] = {};
@@ -319,11 +327,6 @@ void free_all(gba_handle* h) {
   for (int b = 0; b < SLOTS; ++b) {
     cudaFree(h->d_meta[b]);
     cudaFree(h->d_step_scratch[b]);
-    cudaFree(h->d_status[b]);
-    for (int i = 0; i < 2; ++i) {
-      cudaFree(h->d_keys[b][i]);
-      cudaFree(h->d_vals[b][i]);
-    }
     for (cudaEvent_t e : {h->ev_hist[b], h->ev_sorted[b], h->ev_applied[b], h->ev_densed[b]})
       if (e) cudaEventDestroy(e);
   }
@@ -331,11 +334,8 @@ void free_all(gba_handle* h) {
     if (h->h_meta[i]) cudaFreeHost(h->h_meta[i]);
     if (h->meta_ev[i]) cudaEventDestroy(h->meta_ev[i]);
   }
-  for (void* p : {(void*)h->d_rr, (void*)h->d_kl, (void*)h->d_kw, (void*)h->d_scan_status,
-                  (void*)h->d_long_rows, (void*)h->d_long_done, (void*)h->d_items,
-                  (void*)h->d_part_hi, (void*)h->d_part_lo, (void*)h->d_ustart,
-                  (void*)h->d_small_rows})
-    cudaFree(p);
+  for (char* p : h->step_blocks) cudaFree(p);
+  cudaFree(h->d_ustart);
   cudaFree(h->d_err);
   cudaFree(h->d_wtab);
   cudaFree(h->d_acc);
@@ -527,60 +527,60 @@ gba_status grow_hash_tables(gba_handle* h, const std::vector<int64_t>& nbase) {
   return st;
 }
 
+// The step's buffers, for N occurrences and the sort's plan.
 gba_status ensure_step_capacity(gba_handle* h, int64_t N) {
-  if (N > h->n_cap) {
-    sync_all(h);
-    const int64_t cap = std::max<int64_t>(N + N / 4, 4096);
-    h->n_cap = 0;  // until every buffer is there: what a failed allocation leaves serves no step
-    const size_t status_bytes = sort_status_words(cap, MAX_RADIX) * sizeof(unsigned long long);
-    for (int b = 0; b < SLOTS; ++b) {
-      for (int i = 0; i < 2; ++i) {
-        cudaFree(h->d_keys[b][i]);
-        cudaFree(h->d_vals[b][i]);
-        h->d_keys[b][i] = h->d_vals[b][i] = nullptr;
-        GBA_CUDA(h, cudaMalloc(&h->d_keys[b][i], cap * sizeof(uint32_t)));
-        GBA_CUDA(h, cudaMalloc(&h->d_vals[b][i], cap * sizeof(uint32_t)));
-      }
-      cudaFree(h->d_status[b]);
-      h->d_status[b] = nullptr;
-      GBA_CUDA(h, cudaMalloc(&h->d_status[b], status_bytes));
-      GBA_CUDA(h, cudaMemsetAsync(h->d_status[b], 0, status_bytes, h->stream));
+  if (N == 0 || (N <= h->n_cap && h->plan.radix <= h->cap_radix)) return GBA_OK;
+  sync_all(h);
+  const int64_t cap = std::max({N + N / 4, h->n_cap, (int64_t)4096});
+  h->n_cap = 0;  // until every buffer is there: what a failed allocation leaves serves no step
+  h->have_last = false;
+  for (char* p : h->step_blocks) cudaFree(p);
+  h->step_blocks.clear();
+  std::vector<std::pair<void**, size_t>> arrays;
+  auto array = [&](auto*& p, size_t count) {
+    arrays.emplace_back(reinterpret_cast<void**>(&p), (count * sizeof(*p) + 255) & ~(size_t)255);
+  };
+  // look-back words, keys and payloads of the sort
+  for (int b = 0; b < SLOTS; ++b) array(h->d_status[b], sort_status_words(cap, h->plan.radix));
+  array(h->d_scan_status, (size_t)scan_tiles(cap) * 4);
+  const size_t n_cleared = arrays.size();  // epoch 0: of no launch
+  for (int b = 0; b < SLOTS; ++b)
+    for (int i = 0; i < 2; ++i) {
+      array(h->d_keys[b][i], (size_t)cap);
+      array(h->d_vals[b][i], (size_t)cap);
     }
-    // row-kernel buffers: a record per possible row (and one for the totals),
-    // a kept-list entry per occurrence, look-back words per scan tile,
-    // long rows and their chunks
-    for (void* p : {(void*)h->d_rr, (void*)h->d_kl, (void*)h->d_kw, (void*)h->d_scan_status,
-                    (void*)h->d_long_rows, (void*)h->d_long_done, (void*)h->d_items,
-                    (void*)h->d_part_hi, (void*)h->d_part_lo, (void*)h->d_small_rows})
-      cudaFree(p);
-    h->d_rr = nullptr;
-    h->d_kl = nullptr;
-    h->d_kw = h->d_part_hi = h->d_part_lo = nullptr;
-    h->d_scan_status = nullptr;
-    h->d_long_rows = nullptr;
-    h->d_small_rows = nullptr;
-    h->d_long_done = nullptr;
-    h->d_items = nullptr;
-    const int64_t stiles = scan_tiles(cap);
-    const int64_t long_cap = cap / (LONG_ROW + 1) + h->T + 1;
-    const int64_t items_cap = long_items(cap, h->num_sms) + long_cap;
-    int64_t part_floats = 1;  // of the widest range of tables
-    for (const TableState& ts : h->tables)
-      part_floats = std::max(part_floats, long_parts(cap, ts.desc.dim, h->num_sms) * ts.desc.dim);
-    GBA_CUDA(h, cudaMalloc(&h->d_rr, (size_t)(cap + h->T + 1) * sizeof(uint4)));
-    GBA_CUDA(h, cudaMalloc(&h->d_kl, (size_t)cap * sizeof(float*)));
-    GBA_CUDA(h, cudaMalloc(&h->d_kw, (size_t)cap * sizeof(float)));
-    GBA_CUDA(h, cudaMalloc(&h->d_scan_status, (size_t)stiles * 4 * sizeof(unsigned long long)));
-    GBA_CUDA(h, cudaMemsetAsync(h->d_scan_status, 0, (size_t)stiles * 4 * sizeof(unsigned long long),
-                                h->stream));
-    GBA_CUDA(h, cudaMalloc(&h->d_long_rows, (size_t)long_cap * sizeof(uint4)));
-    GBA_CUDA(h, cudaMalloc(&h->d_small_rows, (size_t)long_cap * sizeof(uint4)));
-    GBA_CUDA(h, cudaMalloc(&h->d_long_done, (size_t)long_cap * sizeof(uint32_t)));
-    GBA_CUDA(h, cudaMalloc(&h->d_items, (size_t)items_cap * sizeof(uint2)));
-    GBA_CUDA(h, cudaMalloc(&h->d_part_hi, (size_t)part_floats * sizeof(float)));
-    GBA_CUDA(h, cudaMalloc(&h->d_part_lo, (size_t)part_floats * sizeof(float)));
-    h->n_cap = cap;
+  // row-kernel buffers: a record per possible row (and one for the totals),
+  // a kept-list entry per occurrence (with its weight where weights differ from
+  // 1), long rows and their chunks
+  const int64_t long_cap = cap / (LONG_ROW + 1) + h->T + 1;
+  int64_t part_floats = 1;  // of the widest range of tables
+  for (const TableState& ts : h->tables)
+    part_floats = std::max(part_floats, long_parts(cap, ts.desc.dim, h->num_sms) * ts.desc.dim);
+  array(h->d_rr, (size_t)(cap + h->T + 1));
+  array(h->d_kl, (size_t)cap);
+  array(h->d_kw, h->st.decay != 0 ? (size_t)cap : 1);
+  array(h->d_long_rows, (size_t)long_cap);
+  array(h->d_small_rows, (size_t)long_cap);
+  array(h->d_long_done, (size_t)long_cap);
+  array(h->d_items, (size_t)(long_items(cap, h->num_sms) + long_cap));
+  array(h->d_part_hi, (size_t)part_floats);
+  array(h->d_part_lo, (size_t)part_floats);
+
+  size_t total = 0;
+  for (const auto& x : arrays) total += x.second;
+  const bool apart = total <= ONE_STEP_BLOCK;
+  char* block = nullptr;
+  for (size_t i = 0; i < arrays.size(); ++i) {
+    if (apart || i == 0) {
+      GBA_CUDA(h, cudaMalloc(&block, apart ? arrays[i].second : total));
+      h->step_blocks.push_back(block);
+    }
+    *arrays[i].first = block;
+    if (i < n_cleared) GBA_CUDA(h, cudaMemsetAsync(block, 0, arrays[i].second, h->stream));
+    block += arrays[i].second;
   }
+  h->n_cap = cap;
+  h->cap_radix = h->plan.radix;
   return GBA_OK;
 }
 

@@ -48,7 +48,7 @@ void launch_seg_scan(const StepArgs& a, const SegTable&, const SegTable*, const 
   fake_need(vals, (size_t)a.N * 4);
   fake_need(so.rr, (size_t)(a.N + 1) * sizeof(uint4));
   fake_need(so.kl, (size_t)a.N * 8);
-  fake_need(so.kw, (size_t)a.N * 4);
+  if (a.decay) fake_need(so.kw, (size_t)a.N * 4);
   fake_need(so.status, (size_t)scan_tiles(a.N) * 32);
 }
 void launch_row_apply(const StepArgs&, const RowRange& r, const SegTable*, const SegOut& so, DevStats*,

@@ -103,19 +103,21 @@ def test_a_push_whose_copy_failed_takes_no_place_in_the_buffer(F, kind, nth, eag
     assert h.apply() == 1
 
 
-@pytest.mark.parametrize("nth", range(1, 21))
-def test_a_step_whose_buffers_could_not_grow_is_refused_until_they_can(F, nth):
-    """The n-th of the step's allocations fails: the step is not applied and
-    stays buffered, a smaller one does not run on what is left of the buffers,
-    and the next that finds memory allocates all of them."""
+@pytest.mark.parametrize("n,nth", [(100_000, 1)] + [(10_000, n) for n in range(1, 21)])
+def test_a_step_whose_buffers_could_not_grow_is_refused_until_they_can(F, n, nth):
+    """The n-th allocation of the step's buffers fails: the step is not applied
+    and stays buffered, a smaller one does not run on what is left of the
+    buffers, and the next that finds memory allocates them."""
     h = Handle(F, G=1, max_buf=4, max_ids=200_000, dim=20)
     assert h.push(n=600, ref=True) == B.GBA_OK
     assert h.apply() == 1
-    assert h.push(n=100_000, ref=True) == B.GBA_OK and h.push(n=10, ref=True) == B.GBA_OK
+    assert h.push(n=n, ref=True) == B.GBA_OK and h.push(n=10, ref=True) == B.GBA_OK
     for _ in range(2):
         F.fake_fail(MALLOC, nth)
         assert h.apply() == B.GBA_E_OOM
     assert F.gba_pull_version(h.h) == 1
+    n_sorted = ctypes.c_int64()  # the record of the step before went with its buffers
+    assert F.gba_debug_sorted(h.h, 0, None, None, ctypes.byref(n_sorted)) == B.GBA_E_STATE
     assert [h.apply(), h.apply(), h.apply()] == [1, 1, 0]
 
 
