@@ -323,8 +323,8 @@ gba_status gba_join(gba_handle* h);
 gba_status gba_set_timing(gba_handle* h, int32_t on);
 gba_status gba_kernel_times(gba_handle* h, gba_kernel_times_t* out);
 
-/* gba_set_debug - when on, each step also records the dedup result so that
- * gba_debug_segments can return it (costs one extra write per unique row). */
+/* gba_set_debug - when on, gba_debug_segments returns the dedup result of the
+ * last step (from the records that every step writes). */
 gba_status gba_set_debug(gba_handle* h, int32_t on);
 
 /*

@@ -21,15 +21,17 @@ namespace gba {
 
 namespace {
 
-#ifndef GBA_DENSE_TILE
-#define GBA_DENSE_TILE 2048
-#endif
-constexpr int DT = GBA_DENSE_TILE;       // parameters per tile
-// Stages of DT floats: as many as help the largest updates, or fewer, so that
-// three CTAs leave the kernels of the other streams 107 KB of an SM's shared memory
-// instead of 33, for updates that are short beside them (D x M of at most
-// DENSE_SHORT bytes, and more than one CTA per SM): steps of 1M x 32 gradients 186.1 ->
-// 178.2 us, 2M x 32 305.8 -> 295.8; with 5 stages 64M x 16 took 1% longer.
+constexpr int DT = 2048;                 // parameters per tile
+// Stages of DT floats: as many as help the largest updates, or fewer for updates
+// that are short beside the row path (M gradients of D floats of at most DENSE_SHORT
+// bytes, all M counted, and more than one CTA per SM).  Steps of 0.85M ids x 32 floats
+// and 32 dense gradients, with 8 stages and with 5: 0.13 GB of them 231 and 220 us,
+// 0.26 GB 253 and 242, 0.5 GB 298 and 293, 1 GB 376 and 390, 2 GB 542 and 628, 4 GB
+// 874 and 1,199.  It is not the room in shared memory that the shorter ring leaves to
+// other kernels: three CTAs hold 62,208 of an SM's 65,536 registers, so no block of
+// another kernel is beside them with either ring, and asking for the full shared-memory
+// split with 5 stages changes nothing.  What is left is that fewer copies in flight (123 KB
+// an SM instead of 197) keep the row path's loads waiting less; that was not shown.
 constexpr int STAGES_LONG = 8, STAGES_SHORT = 5;
 constexpr int64_t DENSE_SHORT = 256ll << 20;
 constexpr int CONSUMER_WARPS = 8;        // 256 threads

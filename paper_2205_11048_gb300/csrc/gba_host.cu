@@ -1166,7 +1166,6 @@ int32_t gba_try_apply(gba_handle* h) {
     tb.s1 = ts.s1;
     tb.ver = ts.ver;
     tb.d = ts.desc.dim;
-    tb.t = t;
     tb.key_base = ts.key_base;
     tb.rows = (uint32_t)ts.desc.rows;
     tb.nb = (uint32_t)nbase[t];

@@ -95,8 +95,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // be set up in turn.  On steps of ten kernels of 3 to 20 us that takes about a
 // microsecond off each gap (0.03M ids 61.7 -> 54.5 us a step, 0.85M 209.6 ->
 // 200.2); above CHAIN_MAX_N occurrences the waiting blocks' places on the SMs
-// are worth more than the gaps (5.2M and 131M: 0.7% slower), so those steps'
-// kernels start in the plain order.  Pulls, the copies of pushes and push-time
+// are worth more than the gaps where steps overlap (5.2M: 0.7% slower chained) or
+// are long (131M: the same), so those steps' kernels start in the plain order.  One
+// by one, with the scan's registers that go with it (k_seg_scan), chaining takes
+// 278.1 us against 279.6 at 1.3M, 359.8 against 357.0 at 2M, 425 against 430 at 2.6M
+// and 688 against 701 at 5.2M occurrences x 32 floats.  Pulls, the copies of pushes and push-time
 // dense sums, which come one after another, are always chained (N = 0).
 // A block may thus be resident while the kernel before still writes, so memory that
 // any kernel writes (parameters, tags, descriptions, a caller's ids and gradients) is
@@ -361,6 +364,10 @@ __device__ __forceinline__ void csum_add_w(CSum& c, bool unit, float f, float g)
     csum_add_prod(c, f, g);
 }
 
+// Pause between two looks at an earlier tile's words: spinning takes issue slots from
+// the tiles it waits for.
+constexpr unsigned LOOKBACK_SLEEP_NS = 64;
+
 // Accumulated statistics (device).
 struct DevStats {
   unsigned long long steps, msgs_kept, msgs_dropped, dense_stale_sum, dense_stale_max, pairs,
@@ -417,7 +424,9 @@ void launch_weights(const StepArgs& a, StepScratch sc, DevStats* stats, int n_hi
 
 // ---- the sort of the step's keys
 constexpr int MAX_PASSES = 4;
-// Keys per onesweep tile, and of more than SORT_BIG_N keys twice as many.
+// Keys per onesweep tile, and of more than SORT_BIG_N keys twice as many (a step of
+// 1.3M occurrences with either 279 us, 2M 360 with the smaller tiles and 347 with the
+// larger, 2.6M 434 and 429, 5.2M 718 and 700).
 constexpr int SORT_TILE_KEYS = 2048;
 constexpr int64_t SORT_BIG_N = 1 << 21;
 
@@ -460,15 +469,13 @@ struct SegTable {
   float* s1;
   int32_t* ver;
   int32_t d;
-  int32_t t;
   uint32_t key_base;
   uint32_t rows;  // V of the table
   uint32_t nb;    // first position of its keys in the sorted array, and first occurrence
   uint32_t n;     // how many it has
   float mscale;   // messages over occurrences
-  uint32_t pad;
   OptStep opt;
-  uint32_t pad2;
+  uint32_t pad;
 };
 static_assert(sizeof(SegTable) % 8 == 0, "copied as words, followed by 8-byte values");
 
@@ -502,7 +509,7 @@ struct SegOut {
   uint32_t epoch;              // tag of this launch's look-back words
   uint32_t* ticket;            // scan tile tickets (cleared by K1)
   uint32_t* ustart;            // [T + 1]
-  uint32_t* n_long;            // rows with more than SMALL_MAX kept occurrences (cleared by K1)
+  uint32_t* n_long;            // rows with more than small_limit kept occurrences (cleared by K1)
   uint32_t* n_items;           // chunks of those rows (cleared by K1)
   uint32_t* n_parts;           // chunk-sum slots of rows split into chunks (cleared by K1)
   uint32_t* item_ticket;       // items claimed by warps of the long-row kernel (cleared by K1)
@@ -512,20 +519,17 @@ struct SegOut {
   float* part_hi;              // [n_parts][d] compensated chunk sums
   float* part_lo;
   uint4* small_rows;           // [n_small] (row, first kept, table << 8 | kept count, denominator)
-  uint32_t* n_small;           // rows of LONG_ROW + 1 .. SMALL_MAX kept occurrences (cleared by K1)
+  uint32_t* n_small;           // rows of LONG_ROW + 1 .. small_limit kept occurrences (cleared by K1)
   uint32_t* small_ticket;      // small rows claimed by the long-row kernel (cleared by K1)
 };
 
 // Rows with at most LONG_ROW kept occurrences are applied by k_row_apply,
-// rows of at most SMALL_MAX by one lane group of k_row_long each, longer ones
-// in chunks.
+// rows of at most small_limit (SMALL_MAX, or half of it in ranges of up to 2^23
+// occurrences) by one lane group of k_row_long each, longer ones in chunks.
 constexpr int LONG_ROW = 4;
-constexpr int SMALL_MAX = 64;  // half of that in smaller ranges
+constexpr int SMALL_MAX = 64;
 static_assert(SMALL_MAX < 256, "a small row's count shares a word with its table");
-#ifndef GBA_SCAN_TILE
-#define GBA_SCAN_TILE 2048
-#endif
-constexpr int SCAN_TILE = GBA_SCAN_TILE;  // sorted positions per segment-scan tile
+constexpr int SCAN_TILE = 2048;  // sorted positions per segment-scan tile
 
 int64_t scan_tiles(int64_t N);
 // The most chunks, beside one for each long row, that n occurrences can make, and

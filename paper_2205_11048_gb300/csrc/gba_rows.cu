@@ -20,11 +20,11 @@
 //               longer ones are listed for k_row_long, and lane groups then
 //               sum and apply the rest, the next rows' state and gradients
 //               being loaded while the current ones are computed.
-//  k_row_long   Rows with more kept occurrences: up to SMALL_MAX of them by one
-//               lane group each, longer rows in chunks by one warp each, the
-//               warp's lane groups summing contiguous parts that are merged in
-//               a fixed order; the warp that completes a row's last chunk
-//               merges the chunk sums and applies the row.
+//  k_row_long   Rows with more kept occurrences: up to small_limit of them by
+//               one lane group each, longer rows in chunks of chunk_entries by
+//               one warp each, the warp's lane groups summing contiguous parts
+//               that are merged in a fixed order; the warp that completes a
+//               row's last chunk merges the chunk sums and applies the row.
 //
 // The last two run once per range of consecutive tables of one width and
 // optimizer.  Every summation order is fixed (sorted order, then fixed parts
@@ -111,12 +111,10 @@ __device__ __forceinline__ float row_denominator(int mode, uint32_t c_all, uint3
 // once.  0.85M positions 40 -> 18 us, 5.2M (200 MB of tags) 197 -> 100, 131M in
 // four tables 3.12 -> 1.4 ms.
 // ---------------------------------------------------------------------------
-#ifndef GBA_LOOKBACK_SLEEP_NS
-#define GBA_LOOKBACK_SLEEP_NS 64
-#endif
 // BIG: four blocks per SM at 64 registers; a step whose tiles are resident with
 // three all the same (up to CHAIN_MAX_N positions) is faster with 80 registers
 // (0.85M positions: 185.2 -> 181.8 us a step; 131M with 80 registers: 1.2% slower).
+// At 64, all but one table with unit weights spill 16 to 152 bytes a thread.
 template <bool MULTI, bool CACHED, bool UNIT, bool BIG>
 __global__ void __launch_bounds__(SCAN_THREADS, BIG ? 4 : 3)
     k_seg_scan(StepArgs a, SegTable tb0, const SegTable* tabs_g, SegOut so,
@@ -371,7 +369,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, BIG ? 4 : 3)
 #pragma unroll
           for (int c = 0; c < 4; ++c) mine[c] += (uint32_t)(v[c] & ST_COUNT);
         if (done) break;
-        if (take == 0u && GBA_LOOKBACK_SLEEP_NS > 0) __nanosleep(GBA_LOOKBACK_SLEEP_NS);  // back off while predecessors work
+        if (take == 0u) __nanosleep(LOOKBACK_SLEEP_NS);
         j -= take;
       }
 #pragma unroll
@@ -597,7 +595,7 @@ __host__ __device__ inline int row_lanes(int C, int CPL) {
   return L;
 }
 
-// Kept occurrences per chunk of a row longer than SMALL_MAX, for a range of
+// Kept occurrences per chunk of a row longer than small_limit, for a range of
 // tables with n occurrences whose rows take L lanes: 64 for each of the
 // warp's lane groups (128 for a group of 32), and fewer, down to 32, while there
 // would not be two chunks for every warp that can run: such a step's time is that of
@@ -643,6 +641,12 @@ __device__ __forceinline__ int table_of_row(const uint32_t* ustart, int t0, int 
 // 5.2M ids x 64 floats, 1.6M rows moved, beside the other streams' kernels:
 // 505 -> 361 us against one lane group walking its rows through cp.async
 // stages (24 warps per SM, 200 instructions per row).
+// The register limits below spill in some widths (bytes stored a thread): 12 to 72
+// for Adam's rows of up to 128 floats, 28 to 216 for wider ones in float4 pieces,
+// 80 to 144 for odd widths of 65 to 128.  Whole steps of 0.16M even ids are faster
+// all the same than with the kernels before, which did not spill: 65 floats 199 ->
+// 136 us, 127 214 -> 150, Adam's 256 290 -> 219.  Limits without spills were not
+// measured.
 // ---------------------------------------------------------------------------
 // Widths (multiples of 4) up to which k_row_apply loads the next rows into
 // registers while it computes; wider rows are prefetched into L2 instead and
@@ -875,9 +879,14 @@ __global__ void __launch_bounds__(ROW_THREADS, (CH * CPL <= 4 && !AHEAD) ? 4 : (
 // Bound by the latency of the gathers: eight rows in flight per lane group in
 // registers, their addresses read one round ahead (16 warps per SM).  More
 // warps with fewer rows each were slower (24 warps x 8 rows spill; 32 x 4: 73
-// us against 39 on 0.85M ids x 32 floats).  Chunks grow as rows get narrower,
-// so that every lane group has at least 64 entries to pipeline, and a row's
-// chunk sums are merged by all lane groups.  131M ids x 16 floats in four
+// us against 39 on 0.85M ids x 32 floats).  Chunks grow as rows get narrower, so
+// that a full one gives every lane group 32 to 128 entries to pipeline
+// (chunk_entries), and a row's chunk sums are merged by all lane groups.  Odd
+// widths of more than 64 floats spill at 16 warps (96 to 188 bytes stored a thread
+// up to 128 floats, 160 to 728 above, most for Adam with several tables); whole
+// steps of 0.16M skewed ids are faster than with the kernels before all the same:
+// 129 floats 390 -> 277 us, 255 489 -> 354, Adam's 255 501 -> 374.  Fewer rows in
+// flight without spills were not measured.  131M ids x 16 floats in four
 // tables: 8.95 -> 2.17 ms, 68% of the DRAM bandwidth, against staging in shared
 // memory with 8 warps per SM and one lane group merging the chunk sums.
 // ---------------------------------------------------------------------------
@@ -1035,7 +1044,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 2)
     }
   }
 
-  // ---- 2. rows of LONG_ROW + 1 .. SMALL_MAX kept occurrences, one lane group each
+  // ---- 2. rows of LONG_ROW + 1 .. small_limit kept occurrences, one lane group each
   {
     uint32_t base = n_small ? claim(so.small_ticket, (uint32_t)G) : 0u;
     uint4 sr = base + g < n_small ? so.small_rows[base + g] : make_uint4(0u, 0u, 0u, 0u);

@@ -255,17 +255,15 @@ __global__ void __launch_bounds__(SORT_THREADS)
 // digit order before the look-back, so that few registers live through it (48
 // instead of 80: five blocks per SM instead of three); a short last tile is
 // padded with the largest key, which needs no checks.  Lanes of equal digits find
-// each other through a shared word of lane bits per digit in the first pass, where
-// digits come in no order (975 us against 1,097 with match.any on 131M keys), and
+// each other through a shared word of lane bits per digit (a step that CUB's onesweep
+// ranks with as well) in the first pass, where digits come in no order (975 us against 1,097 with match.any on 131M keys), and
 // by match.any in the later ones, where hot keys come in runs that would meet in
 // one word (1,083 us against 824; ballots per bit 1,123).  Above
 // SORT_BIG_N keys a tile holds 4,096 of them (5.2M keys: 70 us a pass against 89
 // with 2,048).  Digits are 8 bits wide, or up to 9 where that saves a pass: 26-bit
-// keys take three passes.  131M keys: 4 x 1.46 -> 1.12 + 2 x 0.83 ms.
+// keys take three passes.  131M keys: 4 x 1.46 -> 1.12 + 2 x 0.83 ms.  The later
+// passes with 256 counters spill 12 to 16 bytes a thread, with 512 and large tiles 56.
 // ---------------------------------------------------------------------------
-#ifndef GBA_LOOKBACK_SLEEP_NS
-#define GBA_LOOKBACK_SLEEP_NS 64
-#endif
 template <int ITEMS, int RADIX, bool FIRST>
 __global__ void __launch_bounds__(SORT_THREADS, ITEMS == 8 ? 5 : 4)
     k_onesweep(SortPass sp, ErrSink err, int64_t wait_ns) {
@@ -479,7 +477,7 @@ __global__ void __launch_bounds__(SORT_THREADS, ITEMS == 8 ? 5 : 4)
           raise_error(err, ERR_TIMEOUT);
           break;
         }
-        if (GBA_LOOKBACK_SLEEP_NS > 0) __nanosleep(GBA_LOOKBACK_SLEEP_NS);  // back off: spinning takes issue slots from the tiles it waits for
+        __nanosleep(LOOKBACK_SLEEP_NS);
       }
     }
 #pragma unroll
