@@ -304,9 +304,9 @@ def test_hot_row_spanning_many_warps():
 @pytest.mark.parametrize("rule", [None, dict(iota=2, decay=1, lam=0.5)])
 def test_kept_count_boundaries_of_the_row_kernels(dim, rule):
     """Rows whose kept occurrences sit on each side of the row kernels' limits
-    -- 4 (short rows), 32 (one lane group per row) and multiples of the
-    128-occurrence chunks -- against the oracle: all messages kept, stale
-    messages dropped, and geometric weights."""
+    in a step of few occurrences -- 4 (short rows), 32 (one lane group per row)
+    and, for the widest of these, the ends of a chunk -- against the oracle: all
+    messages kept, stale messages dropped, and geometric weights."""
     counts = [1, 2, 4, 5, 6, 31, 32, 33, 64, 127, 128, 129, 130, 255, 256, 257, 300]
     V, M, D = len(counts) + 3, 8, 37
     iota = (rule or {}).get("iota", 1)
@@ -430,6 +430,27 @@ def test_tables_that_share_launches():
 
     run_custom(cfg, [batch(0, [0, 3]), batch(1, [1, 2, 8]), batch(2, [0, 1, 2, 5, 7, 8]), batch(3, []),
                      batch(4, [3, 4, 6])])
+
+
+@pytest.mark.parametrize("M", [3, 20])
+@pytest.mark.parametrize("T", [64, 65, 150])
+def test_more_tables_than_the_histogram_caches(T, M):
+    """Around and above the 64 tables whose bounds the histogram keeps in shared
+    memory, with message offsets that fit there and that do not; widths in runs
+    and alone, tables without ids among them, every row length."""
+    shape = [(5 + 7 * (t % 9), (8, 8, 8, 5, 4)[t % 5], int(t % 11 == 3), int(t % 13 == 6)) for t in range(T)]
+    rng = np.random.default_rng(T + M)
+    cfg = cfg_of(shape, D=5, G=M, iota=1)
+
+    def batch(k):
+        out = []
+        for m in range(M):
+            ids = [np.minimum(rng.geometric(0.3, int(rng.integers(0, 60)) * (t % 7 != 2)) - 1, s[0] - 1)
+                   for t, s in enumerate(shape)]
+            out.append(msg(max(0, k - 2 * (m == 2)), ids, [s[1] for s in shape], 5))
+        return out
+
+    run_custom(cfg, [batch(0), batch(1), batch(2)])
 
 
 @pytest.mark.parametrize("rule", [None, dict(iota=3, decay=1, lam=0.5), dict(iota=1, row_staleness=1)])
@@ -843,6 +864,83 @@ def test_copying_push_of_any_alignment(where, shift, eager):
                       [t for i in range(len(dims)) for t in g.table(i) if t is not None])
         g.close()
     for a, b in zip(*states):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("where", ["device", "pinned"])
+def test_copying_push_of_more_pieces_than_blocks(where):
+    """Arrays of many 16 KB pieces between small ones, each at a byte offset of
+    its own.  In pinned memory the pieces outnumber the 64 blocks that read it,
+    so a block goes on to pieces of later arrays, with other access widths: the
+    state is that of the same message pushed by reference."""
+    gen = torch.Generator(device="cuda").manual_seed(12)
+    dims = [64, 1, 7, 3, 32, 2]
+    ns = [5001, 9, 70, 0, 9003, 1]
+    offs = [0, 16, 8, 4, 1, 3, 0, 0, 2, 16, 7, 5, 4]  # of the arrays in the order they are copied
+    D = 400_003
+    tables = [(60, d, 0, 9003, B.opt_desc(0, 0.01)) for d in dims]
+    ids = [torch.randint(0, 60, (n,), generator=gen, device="cuda") for n in ns]
+    rows = [torch.randn(n, d, generator=gen, device="cuda") for n, d in zip(ns, dims)]
+    dense = torch.randn((D + 3) & ~3, generator=gen, device="cuda")[:D]
+    arrays = [x for pair in zip(ids, rows) for x in pair] + [dense]
+    assert sum(-(-x.numel() * x.element_size() // 16384) for x in arrays) > 3 * 64
+    keep = []
+
+    def placed(x, off):  # the address of x's bytes `off` past an allocation's start
+        raw = x.cpu().numpy().tobytes()
+        buf = torch.zeros(len(raw) + off + 16, dtype=torch.uint8)
+        buf[off:off + len(raw)] = torch.frombuffer(bytearray(raw or b"0"), dtype=torch.uint8)[:len(raw)]
+        buf = buf.pin_memory() if where == "pinned" else buf.to("cuda")
+        keep.append(buf)
+        return buf.data_ptr() + off
+
+    at = [placed(x, o) for x, o in zip(arrays, offs)]
+    torch.cuda.synchronize()
+    states = []
+    for copying in (False, True):
+        g = B.GBA(tables, D, B.opt_desc(1, 0.001), 1, 4, iota=3, seed=4)
+        for _ in range(2):
+            if copying:
+                per = [B.gba_sparse_grad(at[2 * t], n, at[2 * t + 1]) for t, n in enumerate(ns)]
+                assert B.gba_push(g.h, 0, per, at[-1], 1) == B.GBA_OK
+            else:
+                g.push_ref(0, ids, rows, dense, 1)
+            assert g.try_apply() == 1
+        g.sync()
+        states.append([t for t in g.dense() if t is not None] +
+                      [t for i in range(len(dims)) for t in g.table(i) if t is not None])
+        g.close()
+    for a, b in zip(*states):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("by_ref", [False, True])
+def test_eager_dense_with_overlapping_steps(by_ref):
+    """Push-time sums while earlier steps are still running, walked in turns
+    from either end, and rows beside them: the state of the buffered mode with
+    steps one by one, bit for bit."""
+    D, M = 8_000_003, 3
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    grads = [torch.randn((D + 3) & ~3, generator=gen, device="cuda")[:D] for _ in range(M)]
+    ids = [torch.randint(0, 5000, (4000,), generator=gen, device="cuda") for _ in range(M)]
+    rows = [torch.randn(4000, 16, generator=gen, device="cuda") for _ in range(M)]
+    torch.cuda.synchronize()
+    outs = []
+    for eager in (False, True):
+        g = B.GBA([(5000, 16, 0, 4000, B.opt_desc(0, 0.01))], D, B.opt_desc(1, 0.001), M, 4 * M, iota=1,
+                  seed=2)
+        if eager:
+            g.set_eager_dense(True)
+            g.set_overlap(True)
+        for k in range(6):
+            for i in range(M):
+                push = g.push_ref if by_ref else g.push
+                push(max(0, k - i), [ids[(k + i) % M]], [rows[(k + i) % M]], grads[(k * i) % M], 1)
+            assert g.try_apply() == 1
+        g.sync()
+        outs.append([t for t in g.dense() + g.table(0) if t is not None])
+        g.close()
+    for a, b in zip(*outs):
         assert torch.equal(a, b)
 
 
